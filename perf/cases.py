@@ -129,9 +129,15 @@ def draw(rng):
 
 def _basis(d, k, g):
     """U [d, k] fp32: the orthonormal factor of a Gaussian matrix (diag(R) > 0)."""
-    q, r = torch.linalg.qr(torch.randn(d, k, generator=g, device="cuda", dtype=torch.float64))
+    q = _qr(torch.randn(d, k, generator=g, device="cuda", dtype=torch.float64))
+    return q.float().contiguous()
+
+
+def _qr(a):
+    """The orthonormal factor of `a` with diag(R) > 0, factored on the host."""
+    q, r = torch.linalg.qr(a.cpu())
     s = torch.sign(torch.diagonal(r))
-    return (q * torch.where(s == 0, torch.ones_like(s), s)).float().contiguous()
+    return (q * torch.where(s == 0, torch.ones_like(s), s)).cuda()
 
 
 def _ids(case, T, g):
@@ -409,8 +415,8 @@ def _exact_subspace(case, s):
         M += g.T @ Cg[t0:t0 + 8192]
         sq += g.square().sum()
     grad = -2 * M
-    q, r = torch.linalg.qr(U - s["eta"] * (grad - U @ (U.T @ grad)))
-    return {"M": M, "acc": (sq - Cg.square().sum()).reshape(1), "U": q * torch.sign(torch.diagonal(r))}
+    return {"M": M, "acc": (sq - Cg.square().sum()).reshape(1),
+            "U": _qr(U - s["eta"] * (grad - U @ (U.T @ grad)))}
 
 
 def _exact_adamw(case, s):
