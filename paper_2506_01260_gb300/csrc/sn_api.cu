@@ -132,16 +132,32 @@ sn_status sn_basis_create(const float *U, int32_t d, int32_t k, sn_basis_t *out,
     b->k = k;
     b->n_pad = (k + 15) / 16 * 16;
     b->k64 = (k + 63) / 64 * 64;
-    cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaMalloc(&b->u32, sizeof(float) * (size_t)d * k);
-    if (e == cudaSuccess) e = cudaMalloc(&b->u32t, sizeof(float) * (size_t)d * k);
-    if (e == cudaSuccess) e = cudaMalloc(&b->ut16, sizeof(__nv_bfloat16) * (size_t)b->n_pad * d);
-    if (e == cudaSuccess) e = cudaMalloc(&b->up16, sizeof(__nv_bfloat16) * (size_t)d * b->k64);
-    if (e == cudaSuccess) e = cudaMalloc(&b->err, sizeof(unsigned int));
-    if (e == cudaSuccess)
-        e = cudaDeviceGetAttribute(&b->tail_cap, cudaDevAttrMultiProcessorCount, b->device);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-        e = cudaMalloc(&b->tail[i], sizeof(float) * (size_t)b->tail_cap * 128 * b->n_pad);
+    b->kp = sn::simt_padded_columns(k);
+    cudaError_t e = cudaDeviceGetAttribute(&b->tail_cap, cudaDevAttrMultiProcessorCount, b->device);
+    // one allocation, every buffer on a 256-byte boundary of it
+    const size_t dk = sizeof(float) * (size_t)d * k;
+    const size_t tail = sizeof(float) * (size_t)b->tail_cap * 128 * b->n_pad;
+    const size_t bytes[8] = {dk, dk, sizeof(float) * (size_t)((d + 31) / 32 * 32) * b->kp,
+                             sizeof(__nv_bfloat16) * (size_t)b->n_pad * d,
+                             sizeof(__nv_bfloat16) * (size_t)d * b->k64, sizeof(unsigned int), tail,
+                             tail};
+    size_t at[8], total = 0;
+    for (int i = 0; i < 8; ++i) {
+        at[i] = total;
+        total += (bytes[i] + 255) & ~(size_t)255;
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&b->mem, total);
+    if (e == cudaSuccess) {
+        char *m = (char *)b->mem;
+        b->u32 = (float *)(m + at[0]);
+        b->u32t = (float *)(m + at[1]);
+        b->u32p = (float *)(m + at[2]);
+        b->ut16 = (__nv_bfloat16 *)(m + at[3]);
+        b->up16 = (__nv_bfloat16 *)(m + at[4]);
+        b->err = (unsigned int *)(m + at[5]);
+        b->tail[0] = (float *)(m + at[6]);
+        b->tail[1] = (float *)(m + at[7]);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(b->err, 0, sizeof(unsigned int), stream);
     if (e == cudaSuccess) e = sn::prepare_basis(*b, U, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -157,14 +173,7 @@ sn_status sn_basis_destroy(sn_basis_t b)
 {
     if (!b)
         return SN_OK;
-    cudaError_t e = cudaSuccess, e2;
-    if ((e2 = cudaFree(b->u32)) != cudaSuccess) e = e2;
-    if ((e2 = cudaFree(b->u32t)) != cudaSuccess) e = e2;
-    if ((e2 = cudaFree(b->ut16)) != cudaSuccess) e = e2;
-    if ((e2 = cudaFree(b->up16)) != cudaSuccess) e = e2;
-    if ((e2 = cudaFree(b->err)) != cudaSuccess) e = e2;
-    for (int i = 0; i < 2; ++i)
-        if ((e2 = cudaFree(b->tail[i])) != cudaSuccess) e = e2;
+    const cudaError_t e = cudaFree(b->mem);
     delete b;
     return cuda_status(e);
 }
@@ -188,7 +197,7 @@ sn_status sn_compress_fwd(sn_basis_t b, sn_dtype dt, const void *X, const int32_
         return st;
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
-        return cuda_status(sn::simt_compress<float>(*b, (const float *)X, ids, pos, T, seq_len,
+        return cuda_status(sn::simt_compress(*b, (const float *)X, ids, pos, T, seq_len,
                                                     (const float *)tok, vocab, (const float *)pe,
                                                     (float *)C, true, s));
     sn::TcArgs a{(const __nv_bfloat16 *)X, ids, pos, (const __nv_bfloat16 *)tok,
@@ -206,7 +215,7 @@ sn_status sn_decompress_fwd(sn_basis_t b, sn_dtype dt, const void *C, const int3
         return st;
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
-        return cuda_status(sn::simt_decompress<float>(*b, (const float *)C, ids, pos, T, seq_len,
+        return cuda_status(sn::simt_decompress(*b, (const float *)C, ids, pos, T, seq_len,
                                                       (const float *)tok, vocab,
                                                       (const float *)pe, (float *)X, true, s));
     sn::TcArgs a{nullptr, ids, pos, (const __nv_bfloat16 *)tok, (const __nv_bfloat16 *)pe,
@@ -233,7 +242,7 @@ sn_status sn_compress_bwd(sn_basis_t b, sn_dtype dt, const void *G, int64_t T, v
         return SN_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
-        return cuda_status(sn::simt_compress<float>(*b, (const float *)G, nullptr, nullptr, T, 1,
+        return cuda_status(sn::simt_compress(*b, (const float *)G, nullptr, nullptr, T, 1,
                                                     nullptr, 1, nullptr, (float *)C, false, s));
     sn::TcArgs a{(const __nv_bfloat16 *)G, nullptr, nullptr, nullptr, nullptr,
                  (__nv_bfloat16 *)C, T, 1, 1, false};
@@ -259,7 +268,7 @@ sn_status sn_decompress_bwd(sn_basis_t b, sn_dtype dt, const void *C, int64_t T,
         return SN_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
-        return cuda_status(sn::simt_decompress<float>(*b, (const float *)C, nullptr, nullptr, T,
+        return cuda_status(sn::simt_decompress(*b, (const float *)C, nullptr, nullptr, T,
                                                       1, nullptr, 1, nullptr, (float *)G, false,
                                                       s));
     sn::TcArgs a{nullptr, nullptr, nullptr, nullptr, nullptr, (__nv_bfloat16 *)C, T, 1, 1,
@@ -310,7 +319,7 @@ sn_status sn_project_weight(sn_basis_t b, sn_dtype dt, const void *W, int64_t ro
         return SN_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
-        return cuda_status(sn::simt_project<float>(*b, (const float *)W, cols, ld, (float *)W_out,
+        return cuda_status(sn::simt_project(*b, (const float *)W, cols, ld, (float *)W_out,
                                                    (float *)ws, s));
     return cuda_status(sn::tc_project(*b, (const __nv_bfloat16 *)W, cols, ld,
                                       (__nv_bfloat16 *)W_out, ws, s));

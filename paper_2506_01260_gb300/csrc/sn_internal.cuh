@@ -17,6 +17,8 @@ enum : unsigned int {
 // Padded copies of U kept by a basis handle.
 //   u32  [d, k]      fp32, as given (CUDA-core paths, row i = U[i, :])
 //   u32t [k, d]      fp32 transpose (CUDA-core reconstruction, coalesced in d)
+//   u32p [d32/2, kp, 2]  fp32, rows of U in pairs, zero past k and d (d32 = d rounded
+//                    up to 32; CUDA-core compress)
 //   ut16 [n_pad, d]  bf16 U^T, rows >= k zero: B operand of the d -> k contraction
 //   up16 [d, k64]    bf16 U, columns >= k zero: operand of the k -> d expansion
 struct sn_basis {
@@ -24,8 +26,11 @@ struct sn_basis {
     int d, k;
     int n_pad;   // k rounded up to 16 (MMA N of the compress contraction)
     int k64;     // k rounded up to 64 (whole 128-byte swizzle atoms)
+    int kp;      // k rounded up to the CUDA-core compress's columns (u32p)
+    void *mem;   // the one device allocation that every buffer below lies in
     float *u32;
     float *u32t;
+    float *u32p;
     __nv_bfloat16 *ut16;
     __nv_bfloat16 *up16;
     unsigned int *err;
@@ -42,17 +47,15 @@ namespace sn {
 void count_launch(int n = 1);
 
 // ---- CUDA-core kernels (fp32 path) -------------------------------------------
-template <typename E>
-cudaError_t simt_compress(const sn_basis &b, const E *X, const int32_t *ids, const int32_t *pos,
-                          int64_t T, int seq_len, const E *tok, int64_t vocab, const E *pe,
-                          E *C, bool gather, cudaStream_t s);
-template <typename E>
-cudaError_t simt_decompress(const sn_basis &b, const E *C, const int32_t *ids,
-                            const int32_t *pos, int64_t T, int seq_len, const E *tok,
-                            int64_t vocab, const E *pe, E *X, bool gather, cudaStream_t s);
-template <typename E>
-cudaError_t simt_project(const sn_basis &b, const E *W, int64_t cols, int64_t ld, E *W_out,
+cudaError_t simt_compress(const sn_basis &b, const float *X, const int32_t *ids, const int32_t *pos,
+                          int64_t T, int seq_len, const float *tok, int64_t vocab, const float *pe,
+                          float *C, bool gather, cudaStream_t s);
+cudaError_t simt_decompress(const sn_basis &b, const float *C, const int32_t *ids,
+                            const int32_t *pos, int64_t T, int seq_len, const float *tok,
+                            int64_t vocab, const float *pe, float *X, bool gather, cudaStream_t s);
+cudaError_t simt_project(const sn_basis &b, const float *W, int64_t cols, int64_t ld, float *W_out,
                          float *A, cudaStream_t s);
+int simt_padded_columns(int k);   // sn_basis::kp
 
 cudaError_t prepare_basis(sn_basis &b, const float *U, cudaStream_t s);
 

@@ -3,24 +3,18 @@
 //
 // fp32 inputs must match the fp64 definition to ~1e-5 relative, which rules
 // out TF32/bf16 tensor-core inputs; these kernels use fp32 FMA with fp32
-// accumulation in ascending-d order per output.
+// accumulation.  At k = 20 they do 5-10 flops per byte read, so both the FMA
+// pipe (74 TFLOP/s) and HBM bound them: every kernel keeps a register tile per
+// thread (an operand read from shared memory feeds 4-32 FMAs), issues packed
+// two-wide FMAs (fma.rn.f32x2: half the issue slots, each half an ordinary
+// fp32 FMA) and splits the long reduction over d between warps and over a
+// thread-block cluster, whose partial sums meet in shared memory.
 #include <algorithm>
 
 #include "sn_internal.cuh"
 
 namespace sn {
 namespace {
-
-__device__ __forceinline__ float to_f(float v) { return v; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 v) { return __bfloat162float(v); }
-template <typename E> __device__ __forceinline__ E from_f(float v);
-template <> __device__ __forceinline__ float from_f<float>(float v) { return v; }
-template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float v)
-{
-    return __float2bfloat16_rn(v);
-}
-
-constexpr int KMAX = 128;   // largest k a handle accepts
 
 // Row state of a token inside a block: skip (t >= T), compute, or zero (bad id).
 enum : int { ROW_SKIP = 0, ROW_OK = 1, ROW_BAD = 2 };
@@ -55,191 +49,640 @@ __device__ __forceinline__ int token_rows(int64_t t, int64_t T, bool gather,
     return ROW_OK;
 }
 
+// ---- packed fp32 pairs, shared memory, clusters ---------------------------------
+typedef unsigned long long f32x2;   // two fp32, the lower-indexed one in the low half
+
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 pack2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ uint32_t smem_addr(const void *p)
+{
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_4(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the fp32 at shared address `a` of the cluster's CTA `rank`
+__device__ __forceinline__ float ld_cluster(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
+    return v;
+}
+
+// Launch a kernel in clusters of `cluster` CTAs along x.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem,
+                            int cluster, cudaStream_t s, Args... args)
+{
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// CTAs per cluster that share one output tile's reduction: the power of two up
+// to 8 with the least (rounds of the grid) x (steps per CTA + 3 for its start + one
+// for each CTA whose partial sums meet), every CTA keeping at least one step.  Among
+// equal costs, the fewest CTAs.  Measured, with 1 / 2 / 4 / 8 CTAs: projection of
+// [2048, 2048] at k = 20 (16 tiles) 74 / 48 / 33 / 37 us, of [2048, 8192] (64 tiles)
+// 92 / 67 / 72 / 90 us; compress of 8192 x 2048 (256 tiles) 31 / 34 / 35 / 43 us.
+int cluster_split(int64_t tiles, int steps, int64_t slots)
+{
+    int best = 1;
+    int64_t best_cost = -1;
+    for (int c = 1; c <= 8 && c <= steps; c *= 2) {
+        const int64_t rounds = (tiles * c + slots - 1) / slots;
+        const int64_t cost = rounds * ((steps + c - 1) / c + 3 + c);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 // ---- C[t, :] = (X[t, :] - tok[id] - pe[p]) U  (or G U when !GATHER) -----------
-constexpr int CT = 32;          // tokens per block
-constexpr int CDC = 64;         // d-chunk staged in shared memory
-constexpr int CTHREADS = 256;
-constexpr int CQ = CT * KMAX / CTHREADS;
+// A CTA of four warps owns 32 tokens.  WN warps (1, 2 or 4: k <= 32, 64, 128)
+// form a group that covers all k columns of a run of 32-column chunks of d; the
+// groups of a CTA and the CTAs of a cluster take the chunks in turn and add up
+// their partial sums at the end, so even a few tokens occupy many warps.  Per
+// chunk a group loads the 32 x 32 pieces of X, tok and pe (128-byte row
+// segments) into registers a chunk ahead, stores their fp32 difference to
+// shared memory and multiplies it by 32 rows of U (paired copy u32p, by
+// cp.async).  A thread owns 4 tokens x TN columns, each sum kept as two halves
+// (even and odd columns of d) so that both operands of a packed FMA are pairs
+// as they lie in shared memory.  At T = 8192, d = 2048, k = 20 (134 and 67 MB read):
+// 42 us with embeddings (3.3 TB/s) and 30 us without, where one output per thread
+// and one pair of shared loads per FMA took 271 and 239 us.  What bounds it is the
+// issue rate of the 7-8 warps that the registers leave on an SM (0.37 a cycle) and
+// the shared loads: 28 passes per 20 cycles of FMAs, since a pass serves equal
+// addresses only where neighbouring lanes share them.  Tiles of 8 tokens a thread
+// (18 passes) need 255 registers and were slower (48 and 30 us), so were chunks of
+// 16 columns at twice the warps (45 us).
+constexpr int CTM = 4;          // tokens per thread
+constexpr int CTOK = 8 * CTM;   // tokens per CTA
+constexpr int CCH = 32;         // columns of d per chunk
+constexpr int CPITCH = CCH + 4; // floats per staged row: a column's rows fall in distinct banks
+constexpr int CTHREADS = 128;
 
-template <typename E, bool GATHER>
-__global__ void __launch_bounds__(CTHREADS)
-k_simt_compress(const float *__restrict__ U32, int d, int k, const E *__restrict__ X,
-                const int32_t *__restrict__ ids, const int32_t *__restrict__ pos, int64_t T,
-                int seq_len, const E *__restrict__ tok, int64_t vocab,
-                const E *__restrict__ pe, E *__restrict__ C, unsigned int *err)
+struct SimtCompress {
+    const float *up;            // paired copy of U
+    const float *X, *tok, *pe;
+    const int32_t *ids, *pos;
+    float *C;
+    unsigned int *err;
+    int64_t T, vocab;
+    int d, k, seq_len, split;   // split: CTAs per cluster
+};
+
+template <int WN, int TN, bool GATHER>
+__global__ void __launch_bounds__(CTHREADS) k_simt_compress(const SimtCompress p)
 {
-    __shared__ float Rs[CT][CDC + 1];
-    __shared__ float Us[CDC * KMAX];
-    __shared__ int64_t rtok[CT], rpe[CT];
-    __shared__ int rstate[CT];
-    const int tid = threadIdx.x;
-    const int64_t t0 = (int64_t)blockIdx.x * CT;
-    if (tid < CT)
-        rstate[tid] = token_rows(t0 + tid, T, GATHER, ids, pos, seq_len, vocab, pe != nullptr,
-                                 d, &rtok[tid], &rpe[tid], err);
-    float acc[CQ];
+    constexpr int G = CTHREADS / 32 / WN;        // groups per CTA
+    constexpr int GS = 32 * WN;                   // threads per group
+    constexpr int KP = 4 * TN * WN;               // padded columns of U
+    constexpr int NL = CTOK * CCH / 4 / GS;       // 16-byte pieces per thread and operand
+    constexpr int LR = CTOK / NL;                 // rows that one load of the group covers
+    extern __shared__ __align__(16) float sm[];
+    __shared__ int64_t rtok[CTOK], rpe[CTOK];
+    __shared__ int rstate[CTOK];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int group = warp / WN, wcol = warp % WN, gl = tid % GS;
+    const int rank = (int)(blockIdx.x % p.split);
+    const int64_t t0 = (int64_t)(blockIdx.x / p.split) * CTOK;
+    const bool has_pe = GATHER && p.pe != nullptr;
+    if (tid < CTOK)
+        rstate[tid] = token_rows(t0 + tid, p.T, GATHER, p.ids, p.pos, p.seq_len, p.vocab, has_pe,
+                                 p.d, &rtok[tid], &rpe[tid], p.err);
+    __syncthreads();
+
+    float *rb = sm + group * (2 * CTOK * CPITCH);
+    float *ub = sm + G * (2 * CTOK * CPITCH) + group * (2 * CCH * KP);
+    const int lrow = gl / (CCH / 4), lcol = 4 * (gl % (CCH / 4));
+    unsigned rows_ok = 0;                          // this thread's rows that are read
 #pragma unroll
-    for (int q = 0; q < CQ; ++q)
-        acc[q] = 0.f;
-    const int nout = CT * k;
-    for (int i0 = 0; i0 < d; i0 += CDC) {
-        const int dc = min(CDC, d - i0);
-        __syncthreads();
-        for (int e = tid; e < CT * CDC; e += CTHREADS) {
-            const int tl = e / CDC, ii = e % CDC;
-            float r = 0.f;
-            if (ii < dc && rstate[tl] == ROW_OK) {
-                r = to_f(X[(t0 + tl) * d + i0 + ii]);
-                if (GATHER) {
-                    r -= to_f(tok[rtok[tl] + i0 + ii]);
-                    if (pe)
-                        r -= to_f(pe[rpe[tl] + i0 + ii]);
+    for (int u = 0; u < NL; ++u)
+        rows_ok |= (rstate[lrow + LR * u] == ROW_OK ? 1u : 0u) << u;
+
+    float4 xv[NL], tv[GATHER ? NL : 1], pv[GATHER ? NL : 1];
+    auto load = [&](int c) {
+        const int col = c * CCH + lcol;
+        const bool in = col < p.d;                  // d is a multiple of 8
+        const float *x = p.X + (t0 + lrow) * p.d + col;
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            const int row = lrow + LR * u;
+            const bool ok = in && ((rows_ok >> u) & 1u);
+            xv[u] = ok ? __ldcs((const float4 *)(x + (int64_t)(LR * u) * p.d))
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (GATHER) {
+                tv[u] = ok ? __ldg((const float4 *)(p.tok + rtok[row] + col))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (has_pe)
+                    pv[u] = ok ? __ldg((const float4 *)(p.pe + rpe[row] + col))
+                               : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+    };
+    auto load_u = [&](int c, int b) {
+        const float *src = p.up + (int64_t)c * CCH * KP;
+        const uint32_t dst = smem_addr(ub + b * CCH * KP);
+        for (int f = gl; f < CCH * KP / 4; f += GS)
+            cp_async_16(dst + 16 * f, src + 4 * f);
+    };
+
+    f32x2 acc[CTM][TN];
+#pragma unroll
+    for (int m = 0; m < CTM; ++m)
+#pragma unroll
+        for (int n = 0; n < TN; ++n)
+            acc[m][n] = 0ull;
+    const int tg = lane >> 2, cg = lane & 3;        // token lane, column lane
+    const int nch = (p.d + CCH - 1) / CCH, step = p.split * G;
+    int c = rank * G + group;
+    if (c < nch) {
+        load(c);
+        load_u(c, 0);
+    }
+    for (int it = 0; c < nch; ++it, c += step) {
+        const int b = it & 1;
+#pragma unroll
+        for (int u = 0; u < NL; ++u) {
+            float4 r = xv[u];
+            if (GATHER) {
+                r.x -= tv[u].x;
+                r.y -= tv[u].y;
+                r.z -= tv[u].z;
+                r.w -= tv[u].w;
+                if (has_pe) {
+                    r.x -= pv[u].x;
+                    r.y -= pv[u].y;
+                    r.z -= pv[u].z;
+                    r.w -= pv[u].w;
                 }
             }
-            Rs[tl][ii] = r;
+            *(float4 *)(rb + b * CTOK * CPITCH + (lrow + LR * u) * CPITCH + lcol) = r;
         }
-        for (int e = tid; e < dc * k; e += CTHREADS)
-            Us[e] = U32[(int64_t)i0 * k + e];
-        __syncthreads();
+        cp_async_wait_all();
+        if (WN == 1)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "r"(GS) : "memory");
+        if (c + step < nch) {
+            load(c + step);
+            load_u(c + step, b ^ 1);
+        }
+        const float *rt = rb + b * CTOK * CPITCH + tg * CPITCH;
+        const f32x2 *ut = (const f32x2 *)(ub + b * CCH * KP) + (4 * wcol + cg) * TN;
 #pragma unroll
-        for (int q = 0; q < CQ; ++q) {
-            const int o = tid + q * CTHREADS;
-            if (o < nout) {
-                const int tl = o / k, j = o % k;
-                float s = acc[q];
-                for (int ii = 0; ii < dc; ++ii)
-                    s = fmaf(Rs[tl][ii], Us[ii * k + j], s);
-                acc[q] = s;
+        for (int q = 0; q < CCH / 4; ++q) {
+            ulonglong2 r[CTM];
+#pragma unroll
+            for (int m = 0; m < CTM; ++m)
+                r[m] = *(const ulonglong2 *)(rt + 8 * m * CPITCH + 4 * q);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                f32x2 u[TN];
+                const f32x2 *us = ut + (2 * q + h) * KP;
+                if (TN % 2 == 0) {
+#pragma unroll
+                    for (int n = 0; n < TN / 2; ++n) {
+                        const ulonglong2 w = ((const ulonglong2 *)us)[n];
+                        u[2 * n] = w.x;
+                        u[2 * n + 1] = w.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int n = 0; n < TN; ++n)
+                        u[n] = us[n];
+                }
+#pragma unroll
+                for (int m = 0; m < CTM; ++m)
+#pragma unroll
+                    for (int n = 0; n < TN; ++n)
+                        acc[m][n] = fma2(h ? r[m].y : r[m].x, u[n], acc[m][n]);
             }
         }
     }
+
+    // partial sums of the CTA's groups, then of the cluster's CTAs
+    constexpr int RP = KP + 1;
+    __syncthreads();                                // every group is done with its stages
 #pragma unroll
-    for (int q = 0; q < CQ; ++q) {
-        const int o = tid + q * CTHREADS;
-        if (o < nout) {
-            const int tl = o / k, j = o % k;
-            if (rstate[tl] == ROW_OK)
-                C[(t0 + tl) * k + j] = from_f<E>(acc[q]);
-            else if (rstate[tl] == ROW_BAD)
-                C[(t0 + tl) * k + j] = from_f<E>(0.f);
+    for (int m = 0; m < CTM; ++m)
+#pragma unroll
+        for (int n = 0; n < TN; ++n) {
+            const float2 v = unpack2(acc[m][n]);
+            sm[(group * CTOK + tg + 8 * m) * RP + (4 * wcol + cg) * TN + n] = v.x + v.y;
+        }
+    __syncthreads();
+    const int nout = CTOK * p.k;
+    const int per = (nout + p.split - 1) / p.split;
+    if (p.split > 1) {
+        for (int e = tid; e < nout; e += CTHREADS) {
+            const int o = e / p.k * RP + e % p.k;
+            float v = sm[o];
+#pragma unroll
+            for (int g = 1; g < G; ++g)
+                v += sm[g * CTOK * RP + o];
+            sm[o] = v;
+        }
+        cluster_sync();
+    }
+    for (int e = rank * per + tid; e < min(nout, (rank + 1) * per); e += CTHREADS) {
+        const int tl = e / p.k, o = tl * RP + e % p.k;
+        float v = 0.f;
+        if (p.split > 1) {
+            for (int r = 0; r < p.split; ++r)
+                v += ld_cluster(smem_addr(sm + o), r);
+        } else {
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                v += sm[g * CTOK * RP + o];
+        }
+        if (rstate[tl] != ROW_SKIP)
+            p.C[t0 * p.k + e] = rstate[tl] == ROW_OK ? v : 0.f;
+    }
+    if (p.split > 1)
+        cluster_sync();                             // no CTA leaves while its sums are read
+}
+
+// ---- out[r, c] = sum_j L[r, j] R[j, c] (+ pe[p, c] + tok[id, c]) -----------------
+// The reconstruction (L = C, R = U^T) and the projection's second pass
+// (L = U, R = U^T W).  A CTA keeps 128 columns of R in shared memory and walks down
+// the rows; its warps share nothing else, each taking 16 rows at a time (copied to
+// its own piece of shared memory), a thread 8 rows x 8 columns (two 16-byte runs
+// 64 columns apart).  j goes up in order in one fp32 FMA chain per output; a
+// packed FMA takes two adjacent columns and an element of L twice.  At T = 8192,
+// d = 2048, k = 20: 28 us without and 45 us with embeddings (one column and 8 tokens a
+// thread: 40 and 72 us); the projection's second pass to [2048, 8192] 28 us (98).  The
+// FMA pipe is half busy; the rest is the stores and, with embeddings, the T_fixed rows.
+constexpr int ETILE = 128;      // columns per CTA, rows per step of its eight warps
+constexpr int EROWS = 16;       // rows per warp and step
+constexpr int ETHREADS = 256;
+
+struct SimtExpand {
+    const float *L, *R;
+    const float *tok, *pe;
+    const int32_t *ids, *pos;
+    float *out;
+    unsigned int *err;
+    int64_t rows, cols, ldr, ldo, vocab;
+    int k, seq_len;
+};
+
+template <bool EMB>
+__global__ void __launch_bounds__(ETHREADS, 2) k_simt_expand(const SimtExpand p)
+{
+    extern __shared__ __align__(16) float smx[];
+    const int kq = (p.k + 1) & ~1;                  // j in pairs: odd k gets a zero column
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float *rs = smx;                                // [kq][ETILE]
+    float *ls = smx + kq * ETILE + warp * 2 * EROWS * kq;   // [2][EROWS][kq]
+    __shared__ int64_t rtok[EMB ? 2 * ETILE : 1], rpe[EMB ? 2 * ETILE : 1];
+    __shared__ int rstate[2 * ETILE];
+    const int64_t c0 = (int64_t)blockIdx.x * ETILE;
+    const bool has_pe = EMB && p.pe != nullptr;
+    if (p.ldr % 4 == 0) {
+        for (int e = tid; e < p.k * (ETILE / 4); e += ETHREADS) {
+            const int j = e / (ETILE / 4), q = 4 * (e % (ETILE / 4));
+            if (c0 + q < p.cols)                    // cols = ldr here: whole 16 bytes
+                *(float4 *)(rs + j * ETILE + q) =
+                    __ldg((const float4 *)(p.R + (int64_t)j * p.ldr + c0 + q));
+        }
+    } else {
+        for (int e = tid; e < p.k * ETILE; e += ETHREADS) {
+            const int j = e / ETILE, q = e % ETILE;
+            if (c0 + q < p.cols)
+                rs[e] = __ldg(p.R + (int64_t)j * p.ldr + c0 + q);
+        }
+    }
+    if (kq > p.k) {
+        if (tid < ETILE)
+            rs[p.k * ETILE + tid] = 0.f;
+        ls[lane * kq + p.k] = 0.f;
+    }
+    __syncthreads();
+
+    const int rg = lane >> 4, cl = lane & 15;
+    const int64_t ntiles = (p.rows + ETILE - 1) / ETILE;
+    // the next rows of L (4-byte copies: k may be odd) and their table rows, a step ahead
+    auto fetch = [&](int64_t tile, int b) {
+        const int64_t r0 = tile * ETILE + EROWS * warp;
+        const int nrow = (int)max((int64_t)0, min((int64_t)EROWS, p.rows - r0));
+        const float *src = p.L + r0 * p.k;
+        float *dst = ls + b * EROWS * kq;
+        if (kq == p.k) {
+            for (int e = lane; e < nrow * kq; e += 32)
+                cp_async_4(smem_addr(dst + e), src + e);
+        } else {
+            for (int r = 0; r < nrow; ++r)
+                for (int j = lane; j < p.k; j += 32)
+                    cp_async_4(smem_addr(dst + r * kq + j), src + r * p.k + j);
+        }
+        if (lane < EROWS) {
+            const int w = (b * 8 + warp) * EROWS + lane;
+            if (EMB)
+                rstate[w] = token_rows(r0 + lane, p.rows, true, p.ids, p.pos, p.seq_len, p.vocab,
+                                       has_pe, (int)p.cols, &rtok[w], &rpe[w], p.err);
+            else
+                rstate[w] = lane < nrow ? ROW_OK : ROW_SKIP;
+        }
+    };
+    fetch(blockIdx.y, 0);
+    int b = 0;
+    for (int64_t tile = blockIdx.y; tile < ntiles; tile += gridDim.y, b ^= 1) {
+        const int64_t r0 = tile * ETILE + EROWS * warp;
+        const int w0 = (b * 8 + warp) * EROWS;
+        cp_async_wait_all();
+        __syncwarp();                               // this step's rows are staged
+        if (tile + gridDim.y < ntiles)
+            fetch(tile + gridDim.y, b ^ 1);
+        const float *lt = ls + (b * EROWS + 8 * rg) * kq;
+        // With embeddings the 128 columns are taken 64 at a time, so that the T_fixed rows
+        // can be loaded before the products and still fit the registers.
+#pragma unroll
+        for (int h0 = 0; h0 < (EMB ? 2 : 1); ++h0) {
+            constexpr int NH = EMB ? 1 : 2;         // 64-column runs per turn
+            const float *rt = rs + 64 * h0 + 4 * cl;
+            float4 tv[EMB ? 8 : 1];
+            if (EMB) {                              // p.cols = d is a multiple of 8 here
+                const int64_t c = c0 + 64 * h0 + 4 * cl;
+#pragma unroll
+                for (int m = 0; m < 8; ++m) {
+                    const int r = w0 + 8 * rg + m;
+                    tv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (c + 4 <= p.cols && rstate[r] == ROW_OK)
+                        tv[m] = __ldg((const float4 *)(p.tok + rtok[r] + c));
+                }
+            }
+            f32x2 acc[8][2 * NH];
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+#pragma unroll
+                for (int n = 0; n < 2 * NH; ++n)
+                    acc[m][n] = 0ull;
+#pragma unroll 2
+            for (int j = 0; j < kq; j += 2) {
+                float2 l[8];
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+                    l[m] = *(const float2 *)(lt + m * kq + j);
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    ulonglong2 r[NH];
+#pragma unroll
+                    for (int h = 0; h < NH; ++h)
+                        r[h] = *(const ulonglong2 *)(rt + (j + i) * ETILE + 64 * h);
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) {
+                        const float v = i ? l[m].y : l[m].x;
+                        const f32x2 vv = pack2(v, v);
+#pragma unroll
+                        for (int h = 0; h < NH; ++h) {
+                            acc[m][2 * h] = fma2(vv, r[h].x, acc[m][2 * h]);
+                            acc[m][2 * h + 1] = fma2(vv, r[h].y, acc[m][2 * h + 1]);
+                        }
+                    }
+                }
+            }
+#pragma unroll
+            for (int h = 0; h < NH; ++h) {
+                const int64_t c = c0 + 64 * (h0 + h) + 4 * cl;
+                const bool whole = c + 4 <= p.cols;
+                float4 ev[EMB ? 8 : 1];
+                if (EMB && has_pe) {
+#pragma unroll
+                    for (int m = 0; m < 8; ++m) {
+                        const int r = w0 + 8 * rg + m;
+                        if (whole && rstate[r] == ROW_OK)
+                            ev[m] = __ldg((const float4 *)(p.pe + rpe[r] + c));
+                    }
+                }
+#pragma unroll
+                for (int m = 0; m < 8; ++m) {
+                    const int st = rstate[w0 + 8 * rg + m];
+                    if (st == ROW_SKIP)
+                        continue;
+                    const float2 x = unpack2(acc[m][2 * h]), y = unpack2(acc[m][2 * h + 1]);
+                    float4 v = make_float4(x.x, x.y, y.x, y.y);
+                    if (EMB) {
+                        if (has_pe) {
+                            v.x += ev[m].x;
+                            v.y += ev[m].y;
+                            v.z += ev[m].z;
+                            v.w += ev[m].w;
+                        }
+                        v.x += tv[m].x;
+                        v.y += tv[m].y;
+                        v.z += tv[m].z;
+                        v.w += tv[m].w;
+                        if (st == ROW_BAD)
+                            v = make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                    float *o = p.out + (r0 + 8 * rg + m) * p.ldo + c;
+                    if (whole) {
+                        __stcs((float4 *)o, v);
+                    } else {
+                        if (c < p.cols) o[0] = v.x;
+                        if (c + 1 < p.cols) o[1] = v.y;
+                        if (c + 2 < p.cols) o[2] = v.z;
+                    }
+                }
+            }
         }
     }
 }
 
-// ---- X[t, i] = sum_j C[t, j] U[i, j] (+ pe[p, i] + tok[id, i]) -----------------
-constexpr int DT = 8;           // tokens per block
-constexpr int DTHREADS = 256;   // columns per block
+// ---- A = U^T W (fp32 [k, cols]), the projection's first pass ---------------------
+// A warp owns 128 columns of W (a thread four, as two pairs) and JT columns of U;
+// WN warps form a group that covers all k, and the groups of a CTA and the CTAs of
+// a cluster take blocks of eight rows of W in turn.  W goes from HBM straight to
+// registers (eight 512-byte rows a warp, a block ahead); U comes a block ahead by
+// cp.async from the paired copy u32p and is read by broadcast, two rows x two
+// columns a load for 8 packed FMAs.  [2048, 2048] and [2048, 8192] at k = 20: 20 and
+// 36 us, where one thread per column walked all of d with one load of U per FMA, on
+// 16 and 64 CTAs, 1297 and 1339 us.
+constexpr int PROWS = 8;        // rows of W per group and step
+constexpr int PTHREADS = 256;
 
-template <typename E, bool GATHER>
-__global__ void __launch_bounds__(DTHREADS)
-k_simt_decompress(const float *__restrict__ U32T, int d, int k, const E *__restrict__ C,
-                  const int32_t *__restrict__ ids, const int32_t *__restrict__ pos, int64_t T,
-                  int seq_len, const E *__restrict__ tok, int64_t vocab,
-                  const E *__restrict__ pe, E *__restrict__ X, unsigned int *err)
+struct SimtProject {
+    const float *up, *W;
+    float *A;
+    int64_t cols, ld;
+    int d, k, split;
+};
+
+template <int WN, int JT>
+__global__ void __launch_bounds__(PTHREADS) k_simt_project_a(const SimtProject p)
 {
-    __shared__ float Cs[DT][KMAX];
-    __shared__ int64_t rtok[DT], rpe[DT];
-    __shared__ int rstate[DT];
-    const int tid = threadIdx.x;
-    const int i = blockIdx.x * DTHREADS + tid;
-    for (int64_t t0 = (int64_t)blockIdx.y * DT; t0 < T; t0 += (int64_t)gridDim.y * DT) {
-        __syncthreads();
-        if (tid < DT)
-            rstate[tid] = token_rows(t0 + tid, T, GATHER, ids, pos, seq_len, vocab,
-                                     pe != nullptr, d, &rtok[tid], &rpe[tid], err);
-        for (int e = tid; e < DT * k; e += DTHREADS) {
-            const int tl = e / k, j = e % k;
-            const int64_t t = t0 + tl;
-            Cs[tl][j] = t < T ? to_f(C[t * k + j]) : 0.f;
+    constexpr int G = PTHREADS / 32 / WN, KP = WN * JT;
+    constexpr int BROWS = PROWS * G;                // rows of W per CTA and step
+    extern __shared__ __align__(16) float smp[];    // U: [2][BROWS / 2][KP][2]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int group = warp / WN, jg = warp % WN;
+    const int rank = (int)(blockIdx.x % p.split);
+    const int64_t c0 = (int64_t)(blockIdx.x / p.split) * 128, c = c0 + 4 * lane;
+
+    ulonglong2 w[PROWS];
+    auto load_w = [&](int row0) {
+        const float *src = p.W + (int64_t)row0 * p.ld + c;
+#pragma unroll
+        for (int i = 0; i < PROWS; ++i, src += p.ld) {
+            w[i] = make_ulonglong2(0ull, 0ull);
+            if (row0 < p.d) {                       // d is a multiple of 8: all rows or none
+                if (c + 4 <= p.cols)
+                    w[i] = __ldg((const ulonglong2 *)src);
+                else if (c < p.cols)
+                    w[i] = make_ulonglong2(pack2(src[0], c + 1 < p.cols ? src[1] : 0.f),
+                                           pack2(c + 2 < p.cols ? src[2] : 0.f, 0.f));
+            }
         }
-        __syncthreads();
-        if (i >= d)
+    };
+    auto load_u = [&](int row0, int b) {            // u32p is padded to 32 rows past d
+        const int n = min(BROWS, (p.d + 31) / 32 * 32 - row0) * KP / 4;
+        const float *src = p.up + (int64_t)row0 * KP;
+        const uint32_t dst = smem_addr(smp + b * BROWS * KP);
+        for (int f = tid; f < n; f += PTHREADS)
+            cp_async_16(dst + 16 * f, src + 4 * f);
+    };
+    f32x2 acc[JT][2];
+#pragma unroll
+    for (int j = 0; j < JT; ++j)
+        acc[j][0] = acc[j][1] = 0ull;
+    const int stride = BROWS * p.split;
+    int row = rank * BROWS;
+    load_w(row + PROWS * group);
+    load_u(row, 0);
+    for (int it = 0; row < p.d; ++it, row += stride) {
+        const int b = it & 1;
+        cp_async_wait_all();
+        __syncthreads();                            // this step's U is staged, the last one's used up
+        ulonglong2 cur[PROWS];
+#pragma unroll
+        for (int i = 0; i < PROWS; ++i)
+            cur[i] = w[i];
+        if (row + stride < p.d) {
+            load_w(row + stride + PROWS * group);
+            load_u(row + stride, b ^ 1);
+        }
+        if (row + PROWS * group >= p.d)             // past the end: no rows of U are staged
             continue;
-        float acc[DT];
+        const float *ut = smp + b * BROWS * KP + PROWS * group * KP + 2 * jg * JT;
 #pragma unroll
-        for (int tl = 0; tl < DT; ++tl)
-            acc[tl] = 0.f;
-        for (int j = 0; j < k; ++j) {
-            const float u = U32T[(int64_t)j * d + i];
+        for (int i = 0; i < PROWS / 2; ++i) {
 #pragma unroll
-            for (int tl = 0; tl < DT; ++tl)
-                acc[tl] = fmaf(Cs[tl][j], u, acc[tl]);
-        }
-#pragma unroll
-        for (int tl = 0; tl < DT; ++tl) {
-            const int64_t t = t0 + tl;
-            if (rstate[tl] == ROW_OK) {
-                float v = acc[tl];
-                if (GATHER) {
-                    if (pe)
-                        v += to_f(pe[rpe[tl] + i]);
-                    v += to_f(tok[rtok[tl] + i]);
-                }
-                X[t * d + i] = from_f<E>(v);
-            } else if (rstate[tl] == ROW_BAD) {
-                X[t * d + i] = from_f<E>(0.f);
+            for (int j = 0; j < JT; j += 2) {
+                // (U[2i, j], U[2i + 1, j], U[2i, j + 1], U[2i + 1, j + 1])
+                const float4 u = *(const float4 *)(ut + 2 * i * KP + 2 * j);
+                const f32x2 a0 = pack2(u.x, u.x), a1 = pack2(u.y, u.y);
+                const f32x2 b0 = pack2(u.z, u.z), b1 = pack2(u.w, u.w);
+                acc[j][0] = fma2(a0, cur[2 * i].x, acc[j][0]);
+                acc[j][1] = fma2(a0, cur[2 * i].y, acc[j][1]);
+                acc[j + 1][0] = fma2(b0, cur[2 * i].x, acc[j + 1][0]);
+                acc[j + 1][1] = fma2(b0, cur[2 * i].y, acc[j + 1][1]);
+                acc[j][0] = fma2(a1, cur[2 * i + 1].x, acc[j][0]);
+                acc[j][1] = fma2(a1, cur[2 * i + 1].y, acc[j][1]);
+                acc[j + 1][0] = fma2(b1, cur[2 * i + 1].x, acc[j + 1][0]);
+                acc[j + 1][1] = fma2(b1, cur[2 * i + 1].y, acc[j + 1][1]);
             }
         }
     }
-}
-
-// ---- W' = U (U^T W): A = U^T W (fp32 [k, cols]) then W' = U A ----------------
-constexpr int PJ = 16;          // U columns per thread in the first pass
-
-template <typename E>
-__global__ void __launch_bounds__(256)
-k_simt_project_a(const float *__restrict__ U32, int d, int k, const E *__restrict__ W,
-                 int64_t cols, int64_t ld, float *__restrict__ A)
-{
-    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int j0 = blockIdx.y * PJ;
-    if (c >= cols)
-        return;
-    float acc[PJ];
+    // partial sums [G][KP][128] of the groups, then of the cluster's CTAs
+    float *red = smp;
+    __syncthreads();
 #pragma unroll
-    for (int jj = 0; jj < PJ; ++jj)
-        acc[jj] = 0.f;
-    for (int i = 0; i < d; ++i) {
-        const float w = to_f(W[(int64_t)i * ld + c]);
-        const float *u = U32 + (int64_t)i * k + j0;
+    for (int j = 0; j < JT; ++j)
+        *(ulonglong2 *)(red + ((size_t)group * KP + jg * JT + j) * 128 + 4 * lane) =
+            make_ulonglong2(acc[j][0], acc[j][1]);
+    __syncthreads();
+    const int nout = p.k * 128;
+    for (int e = tid; e < nout; e += PTHREADS) {
+        float v = red[e];
 #pragma unroll
-        for (int jj = 0; jj < PJ; ++jj)
-            if (j0 + jj < k)
-                acc[jj] = fmaf(u[jj], w, acc[jj]);
+        for (int g = 1; g < G; ++g)
+            v += red[(size_t)g * KP * 128 + e];
+        if (p.split > 1)
+            red[e] = v;
+        else if (c0 + (e & 127) < p.cols)
+            p.A[(int64_t)(e >> 7) * p.cols + c0 + (e & 127)] = v;
     }
-#pragma unroll
-    for (int jj = 0; jj < PJ; ++jj)
-        if (j0 + jj < k)
-            A[(int64_t)(j0 + jj) * cols + c] = acc[jj];
-}
-
-template <typename E>
-__global__ void __launch_bounds__(256)
-k_simt_project_b(const float *__restrict__ U32, int d, int k, const float *__restrict__ A,
-                 int64_t cols, int64_t ld, E *__restrict__ W_out)
-{
-    const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x;
-    const int i = blockIdx.y;
-    if (c >= cols || i >= d)
-        return;
-    float s = 0.f;
-    for (int j = 0; j < k; ++j)
-        s = fmaf(U32[(int64_t)i * k + j], A[(int64_t)j * cols + c], s);
-    W_out[(int64_t)i * ld + c] = from_f<E>(s);
+    if (p.split > 1) {
+        cluster_sync();
+        const int per = (nout + p.split - 1) / p.split;
+        for (int e = rank * per + tid; e < min(nout, (rank + 1) * per); e += PTHREADS) {
+            float v = 0.f;
+            for (int r = 0; r < p.split; ++r)
+                v += ld_cluster(smem_addr(red + e), r);
+            if (c0 + (e & 127) < p.cols)
+                p.A[(int64_t)(e >> 7) * p.cols + c0 + (e & 127)] = v;
+        }
+        cluster_sync();                             // no CTA leaves while its sums are read
+    }
 }
 
 // ---- padded copies of U ---------------------------------------------------------
-__global__ void k_prepare_basis(const float *__restrict__ U, int d, int k, int n_pad, int k64,
-                                float *__restrict__ u32t, __nv_bfloat16 *__restrict__ ut16,
-                                __nv_bfloat16 *__restrict__ up16)
+__global__ void k_prepare_basis(const float *__restrict__ U, int d, int k, int n_pad, int k64, int kp,
+                                float *__restrict__ u32t, float *__restrict__ u32p,
+                                __nv_bfloat16 *__restrict__ ut16, __nv_bfloat16 *__restrict__ up16)
 {
     const int64_t n_t = (int64_t)k * d, n_ut = (int64_t)n_pad * d, n_up = (int64_t)d * k64;
-    const int64_t n = max(n_t, max(n_ut, n_up));
+    const int64_t n_p = (int64_t)((d + 31) / 32 * 32) * kp;
+    const int64_t n = max(max(n_t, n_p), max(n_ut, n_up));
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
         if (e < n_t) {            // u32t[j, i] = U[i, j]
             const int64_t j = e / d, i = e % d;
             u32t[e] = U[i * k + j];
+        }
+        if (e < n_p) {            // u32p[i / 2, j, i % 2] = U[i, j], zero for j >= k and i >= d
+            const int64_t q = e >> 1, j = q % kp, i = 2 * (q / kp) + (e & 1);
+            u32p[e] = j < k && i < d ? U[i * k + j] : 0.f;
         }
         if (e < n_ut) {           // ut16[j, i] = U[i, j], zero rows j >= k
             const int64_t j = e / d, i = e % d;
@@ -252,51 +695,150 @@ __global__ void k_prepare_basis(const float *__restrict__ U, int d, int k, int n
     }
 }
 
+// Warps per group and columns per thread of the compress, and (times four) of the
+// projection's first pass: the widths they are built for (at k = 20, 41 and 82
+// the padded columns kp = 4 wn tn are 20, 48 and 96).
+void compress_shape(int k, int *wn, int *tn)
+{
+    *wn = k <= 32 ? 1 : k <= 64 ? 2 : 4;
+    const int t = (k + 4 * *wn - 1) / (4 * *wn);
+    *tn = *wn == 1 ? (t == 7 ? 8 : t) : (t <= 6 ? 6 : 8);
+}
+
+template <int WN, int TN>
+cudaError_t launch_compress_f32(SimtCompress p, bool gather, int sms, cudaStream_t s)
+{
+    constexpr int G = CTHREADS / 32 / WN, KP = 4 * TN * WN;
+    constexpr size_t stage = sizeof(float) * G * (2 * CTOK * CPITCH + 2 * CCH * KP);
+    constexpr size_t red = sizeof(float) * G * CTOK * (KP + 1);
+    constexpr size_t smem = stage > red ? stage : red;
+    const int64_t tiles = (p.T + CTOK - 1) / CTOK;
+    const int steps = ((p.d + CCH - 1) / CCH + G - 1) / G;
+    // registers let two (gather) or three CTAs share an SM
+    p.split = cluster_split(tiles, steps, (int64_t)sms * (gather ? 2 : 3));
+    const unsigned grid = (unsigned)(tiles * p.split);
+    const cudaError_t e =
+        gather ? launch_clusters(k_simt_compress<WN, TN, true>, grid, CTHREADS, smem, p.split, s, p)
+               : launch_clusters(k_simt_compress<WN, TN, false>, grid, CTHREADS, smem, p.split, s, p);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <bool EMB>
+cudaError_t launch_expand_f32(const SimtExpand &p, int sms, cudaStream_t s)
+{
+    const int kq = (p.k + 1) & ~1;
+    const int smem = (int)(sizeof(float) * 3 * ETILE * kq);
+    cudaError_t e = cudaFuncSetAttribute(k_simt_expand<EMB>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess)
+        return e;
+    // CTAs per column tile: the least (rounds of the grid) x (row tiles per CTA + 1 for its
+    // copy of R)
+    const int64_t ctiles = (p.cols + ETILE - 1) / ETILE, rtiles = (p.rows + ETILE - 1) / ETILE;
+    const int64_t slots = (int64_t)sms * (smem <= 110 << 10 ? 2 : 1);
+    int64_t best = -1, gy = 1;
+    for (int64_t y = 1; y <= rtiles && y <= 2 * slots; ++y) {
+        const int64_t cost = (ctiles * y + slots - 1) / slots * ((rtiles + y - 1) / y + 1);
+        if (best < 0 || cost < best) {
+            best = cost;
+            gy = y;
+        }
+    }
+    k_simt_expand<EMB><<<dim3((unsigned)ctiles, (unsigned)gy), ETHREADS, smem, s>>>(p);
+    count_launch();
+    return cudaGetLastError();
+}
+
+template <int WN, int JT>
+cudaError_t launch_project_a(SimtProject p, int sms, cudaStream_t s)
+{
+    constexpr int G = PTHREADS / 32 / WN, KP = WN * JT;
+    constexpr size_t stage = sizeof(float) * 2 * PROWS * G * KP, red = sizeof(float) * G * KP * 128;
+    const int64_t tiles = (p.cols + 127) / 128;
+    const int steps = (p.d + PROWS * G - 1) / (PROWS * G);
+    p.split = cluster_split(tiles, steps, sms);
+    const cudaError_t e = launch_clusters(k_simt_project_a<WN, JT>, (unsigned)(tiles * p.split),
+                                          PTHREADS, stage > red ? stage : red, p.split, s, p);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+int sm_count_f32(int device)
+{
+    int n = 0;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || n <= 0)
+        n = 148;
+    return n;
+}
+
 }  // namespace
 
-template <typename E>
-cudaError_t simt_compress(const sn_basis &b, const E *X, const int32_t *ids, const int32_t *pos,
-                          int64_t T, int seq_len, const E *tok, int64_t vocab, const E *pe,
-                          E *C, bool gather, cudaStream_t s)
+int simt_padded_columns(int k)
 {
-    const int64_t blocks = (T + CT - 1) / CT;
-    if (gather)
-        k_simt_compress<E, true><<<(unsigned)blocks, CTHREADS, 0, s>>>(
-            b.u32, b.d, b.k, X, ids, pos, T, seq_len, tok, vocab, pe, C, b.err);
-    else
-        k_simt_compress<E, false><<<(unsigned)blocks, CTHREADS, 0, s>>>(
-            b.u32, b.d, b.k, X, nullptr, nullptr, T, 1, nullptr, 1, nullptr, C, b.err);
-    count_launch();
-    return cudaGetLastError();
+    int wn, tn;
+    compress_shape(k, &wn, &tn);
+    return 4 * wn * tn;
 }
 
-template <typename E>
-cudaError_t simt_decompress(const sn_basis &b, const E *C, const int32_t *ids,
-                            const int32_t *pos, int64_t T, int seq_len, const E *tok,
-                            int64_t vocab, const E *pe, E *X, bool gather, cudaStream_t s)
+cudaError_t simt_compress(const sn_basis &b, const float *X, const int32_t *ids, const int32_t *pos,
+                          int64_t T, int seq_len, const float *tok, int64_t vocab, const float *pe,
+                          float *C, bool gather, cudaStream_t s)
 {
-    const int64_t tiles = (T + DT - 1) / DT;
-    dim3 grid((b.d + DTHREADS - 1) / DTHREADS, (unsigned)std::min<int64_t>(tiles, 65535));
-    if (gather)
-        k_simt_decompress<E, true><<<grid, DTHREADS, 0, s>>>(
-            b.u32t, b.d, b.k, C, ids, pos, T, seq_len, tok, vocab, pe, X, b.err);
-    else
-        k_simt_decompress<E, false><<<grid, DTHREADS, 0, s>>>(
-            b.u32t, b.d, b.k, C, nullptr, nullptr, T, 1, nullptr, 1, nullptr, X, b.err);
-    count_launch();
-    return cudaGetLastError();
+    SimtCompress p{b.u32p, X, tok, pe, ids, pos, C, b.err, T, vocab, b.d, b.k, seq_len, 1};
+    const int sms = sm_count_f32(b.device);
+    int wn, tn;
+    compress_shape(b.k, &wn, &tn);
+    switch (10 * wn + tn) {
+    case 11: return launch_compress_f32<1, 1>(p, gather, sms, s);
+    case 12: return launch_compress_f32<1, 2>(p, gather, sms, s);
+    case 13: return launch_compress_f32<1, 3>(p, gather, sms, s);
+    case 14: return launch_compress_f32<1, 4>(p, gather, sms, s);
+    case 15: return launch_compress_f32<1, 5>(p, gather, sms, s);
+    case 16: return launch_compress_f32<1, 6>(p, gather, sms, s);
+    case 18: return launch_compress_f32<1, 8>(p, gather, sms, s);
+    case 26: return launch_compress_f32<2, 6>(p, gather, sms, s);
+    case 28: return launch_compress_f32<2, 8>(p, gather, sms, s);
+    case 46: return launch_compress_f32<4, 6>(p, gather, sms, s);
+    default: return launch_compress_f32<4, 8>(p, gather, sms, s);
+    }
 }
 
-template <typename E>
-cudaError_t simt_project(const sn_basis &b, const E *W, int64_t cols, int64_t ld, E *W_out,
+cudaError_t simt_decompress(const sn_basis &b, const float *C, const int32_t *ids,
+                            const int32_t *pos, int64_t T, int seq_len, const float *tok,
+                            int64_t vocab, const float *pe, float *X, bool gather, cudaStream_t s)
+{
+    const SimtExpand p{C, b.u32t, tok, pe, ids, pos, X, b.err, T, b.d, b.d, b.d, vocab, b.k, seq_len};
+    const int sms = sm_count_f32(b.device);
+    return gather ? launch_expand_f32<true>(p, sms, s) : launch_expand_f32<false>(p, sms, s);
+}
+
+cudaError_t simt_project(const sn_basis &b, const float *W, int64_t cols, int64_t ld, float *W_out,
                          float *A, cudaStream_t s)
 {
-    dim3 ga((unsigned)((cols + 255) / 256), (b.k + PJ - 1) / PJ);
-    k_simt_project_a<E><<<ga, 256, 0, s>>>(b.u32, b.d, b.k, W, cols, ld, A);
-    dim3 gb((unsigned)((cols + 255) / 256), b.d);
-    k_simt_project_b<E><<<gb, 256, 0, s>>>(b.u32, b.d, b.k, A, cols, ld, W_out);
-    count_launch(2);
-    return cudaGetLastError();
+    const SimtProject a{b.u32p, W, A, cols, ld, b.d, b.k, 1};
+    const int sms = sm_count_f32(b.device);
+    int wn, tn;
+    compress_shape(b.k, &wn, &tn);
+    cudaError_t e;
+    switch (10 * wn + tn) {
+    case 11: e = launch_project_a<1, 4>(a, sms, s); break;
+    case 12: e = launch_project_a<1, 8>(a, sms, s); break;
+    case 13: e = launch_project_a<1, 12>(a, sms, s); break;
+    case 14: e = launch_project_a<1, 16>(a, sms, s); break;
+    case 15: e = launch_project_a<1, 20>(a, sms, s); break;
+    case 16: e = launch_project_a<1, 24>(a, sms, s); break;
+    case 18: e = launch_project_a<1, 32>(a, sms, s); break;
+    case 26: e = launch_project_a<2, 24>(a, sms, s); break;
+    case 28: e = launch_project_a<2, 32>(a, sms, s); break;
+    case 46: e = launch_project_a<4, 24>(a, sms, s); break;
+    default: e = launch_project_a<4, 32>(a, sms, s); break;
+    }
+    if (e != cudaSuccess)
+        return e;
+    const SimtExpand p{b.u32, A, nullptr, nullptr, nullptr, nullptr, W_out, b.err, b.d, cols, cols,
+                       ld, 1, b.k, 1};
+    return launch_expand_f32<false>(p, sms, s);
 }
 
 cudaError_t prepare_basis(sn_basis &b, const float *U, cudaStream_t s)
@@ -305,30 +847,10 @@ cudaError_t prepare_basis(sn_basis &b, const float *U, cudaStream_t s)
                                     cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess)
         return e;
-    k_prepare_basis<<<304, 256, 0, s>>>(U, b.d, b.k, b.n_pad, b.k64, b.u32t, b.ut16, b.up16);
+    k_prepare_basis<<<304, 256, 0, s>>>(U, b.d, b.k, b.n_pad, b.k64, b.kp, b.u32t, b.u32p, b.ut16,
+                                        b.up16);
     count_launch();
     return cudaGetLastError();
 }
-
-template cudaError_t simt_compress<float>(const sn_basis &, const float *, const int32_t *,
-                                          const int32_t *, int64_t, int, const float *, int64_t,
-                                          const float *, float *, bool, cudaStream_t);
-template cudaError_t simt_compress<__nv_bfloat16>(const sn_basis &, const __nv_bfloat16 *,
-                                                  const int32_t *, const int32_t *, int64_t, int,
-                                                  const __nv_bfloat16 *, int64_t,
-                                                  const __nv_bfloat16 *, __nv_bfloat16 *, bool,
-                                                  cudaStream_t);
-template cudaError_t simt_decompress<float>(const sn_basis &, const float *, const int32_t *,
-                                            const int32_t *, int64_t, int, const float *,
-                                            int64_t, const float *, float *, bool, cudaStream_t);
-template cudaError_t simt_decompress<__nv_bfloat16>(const sn_basis &, const __nv_bfloat16 *,
-                                                    const int32_t *, const int32_t *, int64_t,
-                                                    int, const __nv_bfloat16 *, int64_t,
-                                                    const __nv_bfloat16 *, __nv_bfloat16 *, bool,
-                                                    cudaStream_t);
-template cudaError_t simt_project<float>(const sn_basis &, const float *, int64_t, int64_t,
-                                         float *, float *, cudaStream_t);
-template cudaError_t simt_project<__nv_bfloat16>(const sn_basis &, const __nv_bfloat16 *, int64_t,
-                                                 int64_t, __nv_bfloat16 *, float *, cudaStream_t);
 
 }  // namespace sn
