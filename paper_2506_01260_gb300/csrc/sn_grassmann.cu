@@ -10,201 +10,492 @@
 // The retraction is CholeskyQR2: R1 = chol(A^T A), Q1 = A R1^-1, then the
 // same once more on Q1 (the Cholesky factor has a positive diagonal, so Q is
 // the unique QR factor with diag(R) > 0).  The O(d k^2) products run in fp32
-// on the CUDA cores (Gram matrices as per-64-row partial products summed in
-// fp64 without atomics; A R^-1 as a row-by-matrix product), the O(k^3)
-// Cholesky factor and its triangular inverse in fp32 in one block (this GPU's
-// fp64 rate is a small fraction of its fp32 rate).  A is within a small step
+// on the CUDA cores (Gram matrices as per-64-row partial products summed with
+// their rounding errors, without atomics; A R^-1 as a row-by-matrix product), the O(k^3)
+// Cholesky factor and its triangular inverse in fp32 (this GPU's fp64 rate is a
+// small fraction of its fp32 rate).  A is within a small step
 // of orthonormal, so its Gram matrix is near the identity and the second pass
 // removes what the first leaves; it all runs once every K iterations.
-#include "sn_internal.cuh"
+//
+// The whole step is one cooperative kernel, a CTA per 64 rows: its products take a
+// microsecond or two each, so what counts is the chain of dependent stages.  A CTA
+// keeps its rows in shared memory from U and M to U_new and meets the others only
+// in the three Gram matrices, each two grid barriers: partial products out, every
+// CTA sums a slice of the elements, the sums back in.  Each CTA then factors the
+// k x k matrix for itself, which costs less than a third barrier would.  The
+// stages are functions, not inlined, so that the second use of each finds its
+// instructions cached (inlined, the step took 62 us).  At d = 4096, k = 41 it takes 54
+// us, about 20 of them in the two factorisations and 11 in the six barriers; as
+// twelve kernels (the factorisation a chain of k two-barrier steps and a serial
+// substitution in one block, 47 us each) it took 164 us.
+#include <algorithm>
+
+#include "sn_tc.cuh"
 
 namespace sn {
 namespace {
 
-constexpr int kRows = 64;    // rows of A, B per block in the Gram kernel
-constexpr int kMixRows = 4;  // rows per pass of the row-mix kernel
+constexpr int kRows = 64;       // rows of U per CTA (and per Gram partial)
+constexpr int kStepThreads = 512;
+constexpr int kStepWarps = kStepThreads / 32;
 
-// part[blk, a, b] = sum over the block's kRows rows i of A[i, a] B[i, b] (fp32
-// products and sums over 64 rows); A, B fp32 [d, k] row-major.  Each thread
-// owns 4 x 4 tiles of (a, b) pairs: per row 8 shared loads feed 16 FMAs.
-__global__ void __launch_bounds__(256) k_gram_part(const float *__restrict__ A,
-                                                   const float *__restrict__ B, int d, int k,
-                                                   float *__restrict__ part)
+struct StepParams {
+    const float *U, *M;
+    float *Y, *G1, *G2;         // k x k sums of the three Gram matrices
+    float *A, *Q;               // [d, k]: rows of a CTA that owns several blocks
+    float *part;                // [nblk, k, k] partial products
+    unsigned int *bar;          // barrier arrivals, and a flag that a wait gave up (both zeroed)
+    float *U_new;
+    unsigned int *err;
+    int d, k, nblk;
+    float beta, gamma;          // A = U + beta M + gamma U Y
+};
+
+// Every CTA of the grid has arrived `n` times: their writes before it are visible
+// (through L2: read them with __ldcg).  Bounded like every wait of the library; false
+// when it gave up, in which case every CTA leaves.
+__device__ __noinline__ bool grid_barrier(const StepParams &p, unsigned int n)
 {
-    extern __shared__ float sm[];               // [kRows][k4] of A, then of B (k4 = k padded to 4)
-    const int k4 = (k + 3) & ~3;
-    float *sa = sm, *sb = sm + kRows * k4;
-    const int r0 = blockIdx.x * kRows;
-    const int nr = min(kRows, d - r0);
-    for (int e = threadIdx.x; e < kRows * k4; e += blockDim.x) {
-        const int r = e / k4, c = e - r * k4;
-        const bool in = r < nr && c < k;
-        sa[e] = in ? A[(size_t)(r0 + r) * k + c] : 0.f;
-        sb[e] = in ? B[(size_t)(r0 + r) * k + c] : 0.f;
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(p.bar, 1u);
+        const uint64_t t0 = tc::global_ns();
+        volatile unsigned int *bar = p.bar;
+        int o = 1;
+        while (bar[0] < n * gridDim.x) {
+            if (bar[1]) {
+                o = 0;
+                break;
+            }
+            if (tc::global_ns() - t0 > tc::kWaitLimitNs) {
+                bar[1] = 1u;
+                atomicOr(p.err, SN_EBIT_TIMEOUT);
+                o = 0;
+                break;
+            }
+        }
+        __threadfence();
+        ok = o;
     }
     __syncthreads();
-    float *dst = part + (size_t)blockIdx.x * k * k;
-    const int nt = k4 / 4;
-    for (int tl = threadIdx.x; tl < nt * nt; tl += blockDim.x) {
+    return ok != 0;
+}
+
+// dst[r][c] = src[row0 + r, c] for the block's rows, zero past d and k (pitch k4 <=
+// 128).  A warp takes four rows, all its loads in flight before the first store.
+__device__ __forceinline__ void load_rows(float *dst, const float *src, int row0, int d, int k, int k4)
+{
+    constexpr int N = kRows / kStepWarps;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float v[N][4];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int r = row0 + N * warp + i;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = lane + 32 * q;
+            v[i][q] = r < d && c < k ? __ldcg(src + (size_t)r * k + c) : 0.f;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (lane + 32 * q < k4)
+                dst[(N * warp + i) * k4 + lane + 32 * q] = v[i][q];
+}
+__device__ __forceinline__ void store_rows(float *dst, const float *src, int row0, int d, int k, int k4)
+{
+    constexpr int N = kRows / kStepWarps;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int r = N * warp + i;
+        if (row0 + r < d)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (lane + 32 * q < k)
+                    dst[(size_t)(row0 + r) * k + lane + 32 * q] = src[r * k4 + lane + 32 * q];
+    }
+}
+
+// out[a, b] = sum over the 64 staged rows of sa[r][a] sb[r][b].  A thread owns a
+// 4 x 4 tile of (a, b): per row two 16-byte shared loads feed 16 FMAs.  Where the tiles
+// are fewer than the threads, groups of threads take every rg-th row and their
+// sums meet in `red`.
+__device__ __noinline__ void gram(const float *sa, const float *sb, int k, int k4, float *red, float *out)
+{
+    const int nt = k4 / 4, ntile = nt * nt;
+    const int rg = max(1, min(8, kStepThreads / ntile));
+    for (int t0 = 0; t0 < ntile; t0 += kStepThreads) {      // one turn unless k > 88
+        const int tl = t0 + (rg > 1 ? threadIdx.x % ntile : threadIdx.x);
+        const int g = rg > 1 ? threadIdx.x / ntile : 0;
+        const bool mine = tl < ntile && g < rg;
         const int ta = 4 * (tl / nt), tb = 4 * (tl % nt);
         float acc[4][4] = {};
-        for (int r = 0; r < nr; ++r) {
-            const float4 x = *(const float4 *)(sa + r * k4 + ta);
-            const float4 y = *(const float4 *)(sb + r * k4 + tb);
-            const float xa[4] = {x.x, x.y, x.z, x.w}, yb[4] = {y.x, y.y, y.z, y.w};
+        if (mine)
+#pragma unroll 4
+            for (int r = g; r < kRows; r += rg) {
+                const float4 x = *(const float4 *)(sa + r * k4 + ta);
+                const float4 y = *(const float4 *)(sb + r * k4 + tb);
+                const float xa[4] = {x.x, x.y, x.z, x.w}, yb[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        acc[i][j] = fmaf(xa[i], yb[j], acc[i][j]);
+            }
+        if (rg > 1) {
+            if (mine && g > 0)
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    red[((g - 1) * 16 + i) * ntile + tl] = acc[i / 4][i % 4];
+            __syncthreads();
+            if (mine && g == 0)
+                for (int h = 0; h < rg - 1; ++h)
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        acc[i / 4][i % 4] += red[(h * 16 + i) * ntile + tl];
+        }
+        if (mine && g == 0)
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    acc[i][j] = fmaf(xa[i], yb[j], acc[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (ta + i < k && tb + j < k)
-                    dst[(ta + i) * k + tb + j] = acc[i][j];
+                    if (ta + i < k && tb + j < k)
+                        out[(ta + i) * k + tb + j] = acc[i][j];
     }
-}
-
-// out[e] = sum over the nblk blocks of part[blk, e], summed in fp64 and stored
-// in fp32 (e < k*k): four lanes per element, each summing every fourth block,
-// then a shuffle.
-__global__ void __launch_bounds__(256) k_gram_sum(const float *__restrict__ part, int nblk, int kk,
-                                                  float *__restrict__ out)
-{
-    const int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, q = threadIdx.x & 3;
-    double s = 0.0;
-    if (e < kk)
-        for (int b = q; b < nblk; b += 4)
-            s += (double)part[(size_t)b * kk + e];
-    s += __shfl_xor_sync(0xffffffffu, s, 1);
-    s += __shfl_xor_sync(0xffffffffu, s, 2);
-    if (e < kk && q == 0)
-        out[e] = (float)s;
-}
-
-// out[i, :] = alpha A[i, :] + beta B[i, :] + gamma (A[i, :] W)  (W k x k fp32).
-// One thread per column (k <= 128); kMixRows rows of A staged per pass give
-// each thread kMixRows independent accumulations.
-__global__ void __launch_bounds__(128) k_rowmix(const float *__restrict__ A,
-                                                const float *__restrict__ B,
-                                                const float *__restrict__ W, int d, int k,
-                                                float alpha, float beta, float gamma,
-                                                float *__restrict__ out)
-{
-    extern __shared__ float sw[];               // W (k x k), then kMixRows rows of A
-    float *srow = sw + k * k;
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x)
-        sw[e] = W[e];
-    const int j = threadIdx.x;
-    for (int i0 = kMixRows * blockIdx.x; i0 < d; i0 += kMixRows * gridDim.x) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < kMixRows * k; e += blockDim.x) {
-            const int r = e / k;
-            srow[e] = i0 + r < d ? A[(size_t)i0 * k + e] : 0.f;
-        }
-        __syncthreads();
-        if (j < k) {
-            float acc[kMixRows] = {};
-            for (int l = 0; l < k; ++l) {
-                const float w = sw[l * k + j];
-#pragma unroll
-                for (int r = 0; r < kMixRows; ++r)
-                    acc[r] = fmaf(srow[r * k + l], w, acc[r]);
-            }
-#pragma unroll
-            for (int r = 0; r < kMixRows; ++r)
-                if (i0 + r < d) {
-                    const size_t o = (size_t)(i0 + r) * k + j;
-                    out[o] = alpha * srow[r * k + j] + beta * B[o] + gamma * acc[r];
-                }
-        }
-    }
-}
-
-// Rinv = R^-1 for R the upper Cholesky factor of the symmetric positive-definite
-// G (k x k), G = R^T R, in fp32 (G is the Gram matrix of a nearly orthonormal
-// A, within a small step of the identity).  One block of 128 threads, all in
-// shared memory: R in the upper triangle of s, R^-1 transposed in its strictly
-// lower triangle, the diagonal of R^-1 apart.  Sets *bad when a pivot is not
-// positive.
-__global__ void __launch_bounds__(128) k_cholesky_inv(const float *__restrict__ G, int k,
-                                                      float *__restrict__ Rinv, unsigned int *bad)
-{
-    extern __shared__ float sc[];                // k x k, then k (diagonal of R^-1)
-    float *dinv = sc + k * k;
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x)
-        sc[e] = G[e];
     __syncthreads();
+}
+
+// s + v as s (rounded) plus the rounding error added to e
+__device__ __forceinline__ void two_sum(float &s, float &e, float v)
+{
+    const float t = __fadd_rn(s, v), w = __fsub_rn(t, s);
+    e += __fadd_rn(__fsub_rn(s, __fsub_rn(t, w)), __fsub_rn(v, w));
+    s = t;
+}
+
+// This CTA's slice of out[e] = sum over the blocks of part[blk, e]: 32 elements a warp,
+// the warps that are left over sharing out the blocks.  The sums carry their
+// rounding errors along (Knuth's two-sum), so they are as good as fp64 ones rounded
+// once; a chain of fp64 additions took 3 us a slice on this GPU.
+__device__ __noinline__ void sum_slice(const StepParams &p, float *out, float2 *red)
+{
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = 0; j < k; ++j) {
-        // R[j, j] = sqrt(G[j, j] - sum_{l<j} R[l, j]^2), one warp
-        if (warp == 0) {
-            float t = 0.f;
-            for (int l = lane; l < j; l += 32)
-                t = fmaf(sc[l * k + j], sc[l * k + j], t);
-            for (int o = 16; o > 0; o >>= 1)
-                t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) {
-                float v = sc[j * k + j] - t;
-                if (!(v > 0.f)) {
-                    atomicOr(bad, SN_EBIT_NUMERIC);
-                    v = 1.f;
-                }
-                sc[j * k + j] = sqrtf(v);
+    const int kk = p.k * p.k, per = (kk + gridDim.x - 1) / gridDim.x;
+    const int e0 = blockIdx.x * per, n = min(per, kk - e0);
+    const int nch = (n + 31) / 32;
+    const int G = nch > 0 ? max(1, kStepWarps / nch) : 1;
+    for (int c0 = 0; c0 < nch; c0 += kStepWarps / G) {
+        const int ch = c0 + warp / G, g = warp % G, e = 32 * ch + lane;
+        const bool mine = warp / G < kStepWarps / G && e < n;
+        float s = 0.f, err = 0.f;
+        if (mine)
+            for (int b0 = g; b0 < p.nblk; b0 += 8 * G) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)          // eight loads in flight
+                    v[u] = b0 + u * G < p.nblk ? __ldcg(p.part + (size_t)(b0 + u * G) * kk + e0 + e)
+                                               : 0.f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    two_sum(s, err, v[u]);
             }
+        red[warp * 32 + lane] = make_float2(s, err);
+        __syncthreads();
+        if (mine && g == 0) {
+            for (int h = 1; h < G; ++h) {
+                const float2 v = red[(warp + h) * 32 + lane];
+                two_sum(s, err, v.x);
+                err += v.y;
+            }
+            out[e0 + e] = s + err;
         }
         __syncthreads();
-        // R[j, c] = (G[j, c] - sum_{l<j} R[l, j] R[l, c]) / R[j, j], c > j
-        const float rjj = sc[j * k + j];
-        for (int c = j + 1 + threadIdx.x; c < k; c += blockDim.x) {
-            float t = sc[j * k + c];
-            for (int l = 0; l < j; ++l)
-                t = fmaf(-sc[l * k + j], sc[l * k + c], t);
-            sc[j * k + c] = t / rjj;
-        }
-        __syncthreads();
-    }
-    // column c of R^-1 (R x = e_c, x_i = 0 for i > c), kept transposed at
-    // sc[c * k + i] for i < c
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        dinv[c] = 1.f / sc[c * k + c];
-        for (int i = c - 1; i >= 0; --i) {
-            float t = sc[i * k + c] * dinv[c];
-            for (int l = i + 1; l < c; ++l)
-                t = fmaf(sc[i * k + l], sc[c * k + l], t);
-            sc[c * k + i] = -t / sc[i * k + i];
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
-        const int i = e / k, c = e - i * k;
-        Rinv[e] = i < c ? sc[c * k + i] : (i == c ? dinv[c] : 0.f);
     }
 }
 
-// acc += sum(G^2) - sum(Cg^2) over bf16 G [T, d] and Cg [T, k]
-__global__ void k_residual(const __nv_bfloat16 *__restrict__ G, int64_t ng,
-                           const __nv_bfloat16 *__restrict__ Cg, int64_t nc, double *acc)
+// sa[r][:] = alpha sa[r][:] + beta sb[r][:] + gamma (sa[r][:] W) for the 64 staged
+// rows, W [k4][k4] zero-padded; a thread owns RM rows x 4 columns.
+template <int RM>
+__device__ __forceinline__ void row_mix(float *sa, const float *sb, const float *W, int k4, bool whole,
+                                        float beta, float gamma)
 {
-    // squares summed in fp32 over 16 chunks of 8 (128 positive terms) at a
-    // time, then into fp64: this GPU's fp64 rate could not keep up with one
-    // fp64 operation per element
+    const int nc = k4 / 4, t = threadIdx.x;
+    const int r = RM * (t / nc), c = 4 * (t % nc);
+    const bool mine = r < kRows;
+    float acc[RM][4] = {};
+    if (mine) {
+        for (int l = 0; l < k4; l += 4) {
+            float a[RM][4];
+#pragma unroll
+            for (int i = 0; i < RM; ++i) {
+                const float4 v = *(const float4 *)(sa + (r + i) * k4 + l);
+                a[i][0] = v.x, a[i][1] = v.y, a[i][2] = v.z, a[i][3] = v.w;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = *(const float4 *)(W + (l + q) * k4 + c);
+#pragma unroll
+                for (int i = 0; i < RM; ++i) {
+                    acc[i][0] = fmaf(a[i][q], w.x, acc[i][0]);
+                    acc[i][1] = fmaf(a[i][q], w.y, acc[i][1]);
+                    acc[i][2] = fmaf(a[i][q], w.z, acc[i][2]);
+                    acc[i][3] = fmaf(a[i][q], w.w, acc[i][3]);
+                }
+            }
+        }
+        if (whole)
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    acc[i][j] = sa[(r + i) * k4 + c + j] + beta * sb[(r + i) * k4 + c + j] +
+                                gamma * acc[i][j];
+    }
+    __syncthreads();                                 // every row has been read
+    if (mine)
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+            *(float4 *)(sa + (r + i) * k4 + c) =
+                make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    __syncthreads();
+}
+__device__ __noinline__ void mix(float *sa, const float *sb, const float *W, int k4, bool whole,
+                                    float beta, float gamma)
+{
+    if (k4 <= 64)                                    // 32 x 16 threads at most
+        row_mix<2>(sa, sb, W, k4, whole, beta, gamma);
+    else
+        row_mix<4>(sa, sb, W, k4, whole, beta, gamma);
+}
+
+// W[r][c] = G[r, c], zero-padded to [k4][k4]
+__device__ __noinline__ void load_square(float *W, const float *G, int k, int k4)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float v[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = warp + kStepWarps * i, c = lane + 32 * q;
+            v[i][q] = r < k && c < k ? __ldcg(G + r * k + c) : 0.f;
+        }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int r = warp + kStepWarps * i, c = lane + 32 * q;
+            if (r < k4 && c < k4)
+                W[r * k4 + c] = v[i][q];
+        }
+    __syncthreads();
+}
+
+// W = R^-1 for R the upper Cholesky factor of the symmetric positive-definite G
+// (k x k), G = R^T R, in fp32: elimination without square roots, G = L D L^T, with
+// L^-1 collected in the columns already eliminated.  Step j takes m = G[j, i] / G[j, j]
+// times row j from every later row i, in the columns c > j of G (both triangles, so
+// the rule is the same for all) and c < j of L^-1, whose own column j becomes -m.
+// R^-1 = (D^-1/2 L^-1)^T.  Warp w holds rows 8 w .. 8 w + 7 in registers, lane l the
+// columns l + 32 q.  The chain of k dependent steps is what this costs, so a warp
+// eliminates its eight rows by itself, with shuffles, publishes them (`rows`, 2 x 8 x
+// 128 floats, and 1 / D in `inv`), and the later warps then take all eight from their
+// rows at once: one barrier per eight steps.  Flags a pivot that is not positive
+// and goes on with 1.
+template <int KQ>
+__device__ __noinline__ void cholesky_inverse(const float *G, int k, int k4, float *rows,
+                                                 float *inv, float *W, unsigned int *err)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int np = (k + 7) / 8;                      // panels, one per warp
+    float v[8][KQ];                                  // rows past k are the identity's
+    float dinv = 1.f;                                // lane i < 8: 1 / sqrt(D) of row 8 warp + i
+    bool bad = false;
+    if (warp < np) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int q = 0; q < KQ; ++q) {
+                const int r = 8 * warp + i, c = lane + 32 * q;
+                v[i][q] = r < k && c < k ? __ldcg(G + r * k + c) : (r == c ? 1.f : 0.f);
+            }
+    }
+    for (int t = 0; t < np; ++t) {
+        float *rt = rows + (t & 1) * 8 * 128;        // two buffers: one barrier per panel
+        float *it = inv + (t & 1) * 8;
+        if (warp == t) {
+            const int l0 = 8 * (t & 3);              // its columns: lanes l0 .. l0 + 7, q = t / 4
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                float x = v[j][0];
+#pragma unroll
+                for (int q = 1; q < KQ; ++q)
+                    x = t / 4 == q ? v[j][q] : x;
+                float pv = __shfl_sync(0xffffffffu, x, l0 + j);
+                bad = bad || !(pv > 0.f);
+                pv = pv > 0.f ? pv : 1.f;
+                const float r = __frcp_rn(pv);
+                if (lane == j)
+                    dinv = pv;
+                x *= r;
+#pragma unroll
+                for (int i = j + 1; i < 8; ++i) {
+                    const float m = __shfl_sync(0xffffffffu, x, l0 + i);
+#pragma unroll
+                    for (int q = 0; q < KQ; ++q)
+                        v[i][q] = lane + 32 * q == 8 * t + j ? -m : fmaf(-m, v[j][q], v[i][q]);
+                }
+                if (lane == 0)
+                    it[j] = r;
+#pragma unroll
+                for (int q = 0; q < KQ; ++q)
+                    rt[j * 128 + lane + 32 * q] = v[j][q];
+            }
+            dinv = 1.f / sqrtf(dinv);
+        }
+        __syncthreads();
+        if (warp > t && warp < np) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float r = it[j];
+                float s[KQ];
+#pragma unroll
+                for (int q = 0; q < KQ; ++q)
+                    s[q] = rt[j * 128 + lane + 32 * q];
+                const float4 a = *(const float4 *)(rt + j * 128 + 8 * warp);
+                const float4 b = *(const float4 *)(rt + j * 128 + 8 * warp + 4);
+                const float m[8] = {a.x * r, a.y * r, a.z * r, a.w * r, b.x * r, b.y * r, b.z * r, b.w * r};
+#pragma unroll
+                for (int q = 0; q < KQ; ++q) {
+                    const bool own = lane + 32 * q == 8 * t + j;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        v[i][q] = own ? -m[i] : fmaf(-m[i], s[q], v[i][q]);
+                }
+            }
+        }
+    }
+    if (bad && lane == 0 && blockIdx.x == 0)
+        atomicOr(err, SN_EBIT_NUMERIC);
+    __syncthreads();
+    // W[l][c] = L^-1[c][l] / sqrt(D[c]), zero-padded: row r of L^-1 is column r of W
+    for (int e = threadIdx.x; e < k4 * (k4 - k); e += kStepThreads)
+        W[(e / (k4 - k)) * k4 + k + e % (k4 - k)] = 0.f;
+    if (warp < np)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = 8 * warp + i;
+            const float f = __shfl_sync(0xffffffffu, dinv, i);
+            if (r < k)
+#pragma unroll
+                for (int q = 0; q < KQ; ++q) {
+                    const int l = lane + 32 * q;
+                    if (l < k4)
+                        W[l * k4 + r] = l <= r ? (l < r ? v[i][q] : 1.f) * f : 0.f;
+                }
+        }
+    __syncthreads();
+}
+
+template <int KQ>                                    // ceil(k / 32)
+__global__ void __launch_bounds__(kStepThreads, 1) k_grassmann_step(StepParams p)
+{
+    extern __shared__ __align__(16) float sm[];
+    __shared__ __align__(16) float rows[2 * 8 * 128];
+    __shared__ float inv[2 * 8];
+    const int k = p.k, k4 = (k + 3) & ~3, kk = k * k;
+    float *sa = sm, *sb = sa + kRows * k4, *W = sb + kRows * k4;
+    float *red = W + k4 * k4;                        // sums of the Gram groups and of the slices
+    const bool one = p.nblk <= (int)gridDim.x;       // a block of rows per CTA, kept in sa
+    unsigned int nbar = 0;
+    auto reduce = [&](float *out) {                  // out = the sum of all partial products
+        if (!grid_barrier(p, ++nbar))
+            return false;
+        sum_slice(p, out, (float2 *)red);
+        return grid_barrier(p, ++nbar);
+    };
+    // Y = U^T M
+    for (int blk = blockIdx.x; blk < p.nblk; blk += gridDim.x) {
+        load_rows(sa, p.U, blk * kRows, p.d, k, k4);
+        load_rows(sb, p.M, blk * kRows, p.d, k, k4);
+        __syncthreads();
+        gram(sa, sb, k, k4, red, p.part + (size_t)blk * kk);
+    }
+    if (!reduce(p.Y))
+        return;
+    // A = U + beta M + gamma U Y, and A^T A
+    load_square(W, p.Y, k, k4);
+    for (int blk = blockIdx.x; blk < p.nblk; blk += gridDim.x) {
+        if (!one) {
+            load_rows(sa, p.U, blk * kRows, p.d, k, k4);
+            load_rows(sb, p.M, blk * kRows, p.d, k, k4);
+            __syncthreads();
+        }
+        mix(sa, sb, W, k4, true, p.beta, p.gamma);
+        if (!one)
+            store_rows(p.A, sa, blk * kRows, p.d, k, k4);
+        gram(sa, sa, k, k4, red, p.part + (size_t)blk * kk);
+    }
+    if (!reduce(p.G1))
+        return;
+    // Q1 = A R1^-1, and Q1^T Q1
+    cholesky_inverse<KQ>(p.G1, k, k4, rows, inv, W, p.err);
+    for (int blk = blockIdx.x; blk < p.nblk; blk += gridDim.x) {
+        if (!one) {
+            load_rows(sa, p.A, blk * kRows, p.d, k, k4);
+            __syncthreads();
+        }
+        mix(sa, sb, W, k4, false, 0.f, 1.f);
+        if (!one)
+            store_rows(p.Q, sa, blk * kRows, p.d, k, k4);
+        gram(sa, sa, k, k4, red, p.part + (size_t)blk * kk);
+    }
+    if (!reduce(p.G2))
+        return;
+    // U_new = Q1 R2^-1
+    cholesky_inverse<KQ>(p.G2, k, k4, rows, inv, W, p.err);
+    for (int blk = blockIdx.x; blk < p.nblk; blk += gridDim.x) {
+        if (!one) {
+            load_rows(sa, p.Q, blk * kRows, p.d, k, k4);
+            __syncthreads();
+        }
+        mix(sa, sb, W, k4, false, 0.f, 1.f);
+        store_rows(p.U_new, sa, blk * kRows, p.d, k, k4);
+    }
+}
+
+// acc += sum(G^2) - sum(Cg^2) over bf16 G [T, d] and Cg [T, k].  Bound by the read of
+// G: eight 16-byte loads in flight per thread, four CTAs per SM (T = 16384, d = 4096:
+// 25 us, 5.3 TB/s; with four loads in flight 35 us).  The squares (128 positive terms at
+// a time) are summed in fp32 and then added up in fp64, since this GPU's fp64 rate
+// could not keep up with one fp64 operation per element.
+constexpr int kResLoads = 8;
+
+__global__ void __launch_bounds__(256, 4) k_residual(const __nv_bfloat16 *__restrict__ G, int64_t ng,
+                                                     const __nv_bfloat16 *__restrict__ Cg, int64_t nc,
+                                                     double *acc)
+{
     double s = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t n8 = ng / 8;
-    for (int64_t e0 = t0; e0 < n8; e0 += 16 * stride) {
+    for (int64_t e0 = t0; e0 < n8; e0 += 2 * kResLoads * stride) {
         float f = 0.f;
-        for (int64_t e1 = e0; e1 < e0 + 16 * stride && e1 < n8; e1 += 4 * stride) {
-            uint4 w[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u)     // four 16-byte loads in flight
+        for (int h = 0; h < 2; ++h) {
+            const int64_t e1 = e0 + h * kResLoads * stride;
+            uint4 w[kResLoads];
+#pragma unroll
+            for (int u = 0; u < kResLoads; ++u)
                 w[u] = e1 + u * stride < n8 ? __ldg((const uint4 *)G + e1 + u * stride)
                                             : make_uint4(0, 0, 0, 0);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < kResLoads; ++u) {
                 const uint32_t ws[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -238,13 +529,12 @@ __global__ void k_residual(const __nv_bfloat16 *__restrict__ G, int64_t ng,
     }
 }
 
-int grid_of(int64_t n, int block)
+int sm_count()
 {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t want = (n + block - 1) / block;
-    return (int)(want < 4 * sms ? (want > 0 ? want : 1) : 4 * sms);
+    return sms;
 }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -254,13 +544,15 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 cudaError_t grassmann_residual(const sn_basis &b, const __nv_bfloat16 *G,
                                const __nv_bfloat16 *Cg, int64_t T, double *acc, cudaStream_t s)
 {
-    k_residual<<<grid_of(T * b.d / 8, 256), 256, 0, s>>>(G, T * b.d, Cg, T * b.k, acc);
+    const int64_t want = (T * b.d / 8 + 255) / 256;
+    const int grid = (int)std::min<int64_t>(std::max<int64_t>(want, 1), 4 * sm_count());
+    k_residual<<<grid, 256, 0, s>>>(G, T * b.d, Cg, T * b.k, acc);
     count_launch();
     return cudaGetLastError();
 }
 
-// workspace: Y, G1, G2, R1^-1, R2^-1 (k x k fp32 each) | A, Q1 (d x k fp32
-// each) | Gram partials (one k x k fp32 block per kRows rows)
+// workspace: Y, G1, G2 and the barrier (k x k fp32 each, two spare ones) | A, Q1
+// (d x k fp32 each) | Gram partials (one k x k fp32 block per kRows rows)
 size_t grassmann_step_workspace(const sn_basis &b)
 {
     const size_t kk = align256(sizeof(float) * (size_t)b.k * b.k);
@@ -272,46 +564,54 @@ size_t grassmann_step_workspace(const sn_basis &b)
 cudaError_t grassmann_step(const sn_basis &b, const float *M, int K, float eta, float *U_new,
                            void *workspace, cudaStream_t s)
 {
-    const int d = b.d, k = b.k;
+    const int d = b.d, k = b.k, k4 = (k + 3) & ~3;
     const size_t kk = align256(sizeof(float) * (size_t)k * k);
     const size_t dk = align256(sizeof(float) * (size_t)d * k);
     char *w = (char *)workspace;
-    float *Y = (float *)w, *G1 = (float *)(w + kk), *G2 = (float *)(w + 2 * kk);
-    float *R1i = (float *)(w + 3 * kk), *R2i = (float *)(w + 4 * kk);
-    float *A = (float *)(w + 5 * kk), *Q1 = (float *)(w + 5 * kk + dk);
-    float *part = (float *)(w + 5 * kk + 2 * dk);
-    const int nblk = (d + kRows - 1) / kRows;
-    const size_t gram_smem = sizeof(float) * 2 * kRows * ((k + 3) & ~3);
-    const size_t mix_smem = sizeof(float) * ((size_t)k * k + (size_t)kMixRows * k);
-    const size_t chol_smem = sizeof(float) * ((size_t)k * k + k);
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_gram_part, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)gram_smem)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_rowmix, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)mix_smem)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(k_cholesky_inv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)chol_smem)) != cudaSuccess)
-        return e;
-    const int mix_grid = grid_of((int64_t)(d + kMixRows - 1) / kMixRows * 128, 128);
-    const int sum_grid = (4 * k * k + 255) / 256;
-    auto gram = [&](const float *X, const float *Z, float *out) {
-        k_gram_part<<<nblk, 256, gram_smem, s>>>(X, Z, d, k, part);
-        k_gram_sum<<<sum_grid, 256, 0, s>>>(part, nblk, k * k, out);
-    };
-    // Y = U^T M;  A = U - eta * (c M - U (c Y)) with c = -2 / K
+    // A = U - eta * (c M - U (c Y)) with c = -2 / K
     const double c = -2.0 / K;
-    gram(b.u32, M, Y);
-    k_rowmix<<<mix_grid, 128, mix_smem, s>>>(b.u32, M, Y, d, k, 1.f, (float)(-eta * c),
-                                             (float)(eta * c), A);
-    // CholeskyQR2: Q = A R^-1 with R = chol(A^T A), twice
-    gram(A, A, G1);
-    k_cholesky_inv<<<1, 128, chol_smem, s>>>(G1, k, R1i, b.err);
-    k_rowmix<<<mix_grid, 128, mix_smem, s>>>(A, A, R1i, d, k, 0.f, 0.f, 1.f, Q1);
-    gram(Q1, Q1, G2);
-    k_cholesky_inv<<<1, 128, chol_smem, s>>>(G2, k, R2i, b.err);
-    k_rowmix<<<mix_grid, 128, mix_smem, s>>>(Q1, Q1, R2i, d, k, 0.f, 0.f, 1.f, U_new);
-    count_launch(12);
-    return cudaGetLastError();
+    StepParams p;
+    p.U = b.u32;
+    p.M = M;
+    p.Y = (float *)w;
+    p.G1 = (float *)(w + kk);
+    p.G2 = (float *)(w + 2 * kk);
+    p.bar = (unsigned int *)(w + 3 * kk);
+    p.A = (float *)(w + 5 * kk);
+    p.Q = (float *)(w + 5 * kk + dk);
+    p.part = (float *)(w + 5 * kk + 2 * dk);
+    p.U_new = U_new;
+    p.err = b.err;
+    p.d = d;
+    p.k = k;
+    p.nblk = (d + kRows - 1) / kRows;
+    p.beta = (float)(-eta * c);
+    p.gamma = (float)(eta * c);
+    // rows of U (A, Q1) and M, a k x k matrix, the Gram groups' sums
+    const size_t smem = sizeof(float) * (2 * (size_t)kRows * k4 + (size_t)k4 * k4 + 16 * kStepThreads);
+    void (*const kernels[4])(StepParams) = {k_grassmann_step<1>, k_grassmann_step<2>,
+                                            k_grassmann_step<3>, k_grassmann_step<4>};
+    void (*const kernel)(StepParams) = kernels[(k - 1) / 32];
+    cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(p.bar, 0, 2 * sizeof(unsigned int), s);
+    if (e != cudaSuccess)
+        return e;
+    // cooperative: the CTAs wait for one another, so all are resident (one per SM)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::min(p.nblk, sm_count()));
+    cfg.blockDim = dim3(kStepThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, kernel, p);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace sn

@@ -508,21 +508,31 @@ __global__ void __launch_bounds__(256) k_transpose_pad(const __nv_bfloat16 *__re
                                                       int k, int n_pad, int64_t Tp,
                                                       __nv_bfloat16 *__restrict__ CgT)
 {
-    // 64 tokens per block through shared memory: their k-wide rows are one
-    // contiguous run of Cg (coalesced reads), each output row j gets 64
-    // consecutive tokens (128-byte writes); the row pitch of 130 elements keeps
-    // the column reads on distinct banks.  k <= 128.
+    // 64 tokens per block through shared memory: a warp reads eight k-wide rows
+    // (adjacent, so coalesced; all eight in flight), each output row j gets 64
+    // consecutive tokens (128-byte writes, two tokens a thread); the row pitch of 130
+    // elements keeps the column reads on distinct banks.  k <= 128.  3.8 us for 16384
+    // tokens at k = 41 (10 us with a division per element).
     __shared__ __nv_bfloat16 tile[64][130];
+    griddep_launch_dependents();      // the contraction's set-up may overlap this kernel
     const int64_t t0 = (int64_t)blockIdx.x * 64;
-    const int nt = (int)(T - t0 < 64 ? (T - t0 > 0 ? T - t0 : 0) : 64);
-    for (int f = threadIdx.x; f < 64 * k; f += blockDim.x) {
-        const int tl = f / k, j = f - tl * k;
-        tile[tl][j] = tl < nt ? Cg[t0 * k + f] : __float2bfloat16_rn(0.f);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
+    for (int j = lane; j < k; j += 32) {
+        __nv_bfloat16 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            v[i] = t0 + 8 * warp + i < T ? Cg[(t0 + 8 * warp + i) * k + j] : zero;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            tile[8 * warp + i][j] = v[i];
     }
     __syncthreads();
-    for (int f = threadIdx.x; f < n_pad * 64; f += blockDim.x) {
-        const int j = f >> 6, t = f & 63;
-        CgT[(int64_t)j * Tp + t0 + t] = j < k ? tile[t][j] : __float2bfloat16_rn(0.f);
+    for (int j = warp; j < n_pad; j += 8) {
+        __nv_bfloat162 v;
+        v.x = j < k ? tile[2 * lane][j] : zero;
+        v.y = j < k ? tile[2 * lane + 1][j] : zero;
+        *(__nv_bfloat162 *)(CgT + (int64_t)j * Tp + t0 + 2 * lane) = v;
     }
 }
 

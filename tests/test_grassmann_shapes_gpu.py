@@ -1,0 +1,57 @@
+"""The subspace update at the edges of its kernels' tiles, against the fp64 oracle.
+
+The step runs a CTA per 64 rows of U with 4 x 4 register tiles of the k x k products,
+shared by groups of threads for small k; past one CTA per SM (152 x 64 rows) a CTA
+owns several blocks of rows.  The accumulation transposes Cg 64 tokens at a time.
+Bars: those of the update's other tests (1e-4 relative for the step, U^T U = I to
+1e-5, 1e-2 for M, 1e-3 for the residual).
+"""
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import dev, widen
+from paper_2506_01260_gb300 import workloads as W
+from test_grassmann_gpu import basis_and_grads, grassmann_oracle, rel
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,k", [(16, 1), (64, 4), (72, 5), (128, 33), (200, 64), (264, 65),
+                                 (1000, 89), (520, 128), (12008, 8), (9800, 41)])
+def test_step_shapes(sn, d, k):
+    g = grassmann_oracle()
+    rng = np.random.default_rng(d + k)
+    U32 = W.orthonormal_basis(d, k, rng).astype(np.float32)
+    # any M has a tangent part; a step of about a tenth of the basis
+    M32 = (U32 @ rng.standard_normal((k, k)) + rng.standard_normal((d, k)) / np.sqrt(d)).astype(np.float32)
+    eta = 0.1 / (2.0 * np.linalg.norm(M32.astype(np.float64), 2) / 3)
+    basis = sn.Basis(dev(U32))
+    U1 = sn.sn_grassmann_step(basis, dev(M32), 3, eta)
+    U2 = sn.sn_grassmann_step(basis, dev(M32), 3, eta)
+    sn.sn_check_errors(basis)
+    assert torch.equal(U1, U2)                       # no order of arrival in the sums
+    got = U1.cpu().numpy().astype(np.float64)
+    ref = g.step(U32.astype(np.float64), M32.astype(np.float64), 3, eta)
+    assert rel(got, ref) <= 1e-4
+    assert np.max(np.abs(got.T @ got - np.eye(k))) <= 1e-5
+    basis.destroy()
+
+
+@pytest.mark.parametrize("d,k,T", [(128, 7, 1), (256, 33, 63), (264, 64, 65), (512, 127, 129),
+                                   (136, 2, 40000)])
+def test_accumulate_shapes(sn, d, k, T):
+    g = grassmann_oracle()
+    U32, (Gb,) = basis_and_grads(sn, d, k, T, 1, seed=T + k)
+    basis = sn.Basis(dev(U32))
+    G = dev(Gb)
+    Cg = sn.sn_compress_bwd(basis, G)
+    M = torch.zeros(d, k, dtype=torch.float32, device="cuda")
+    acc = torch.zeros(1, dtype=torch.float64, device="cuda")
+    sn.sn_grassmann_accumulate(basis, G, Cg, M)
+    sn.sn_grassmann_residual(basis, G, Cg, acc)
+    sn.sn_check_errors(basis)
+    G64, U64 = widen(Gb), U32.astype(np.float64)
+    assert rel(M.cpu().numpy().astype(np.float64), g.accumulate(np.zeros((d, k)), G64, U64)) <= 1e-2
+    assert abs(acc.item() - g.residual(G64, U64)) <= 1e-3 * np.sum(G64 * G64)
+    basis.destroy()
