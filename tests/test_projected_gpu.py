@@ -119,3 +119,30 @@ def test_projected_argument_errors(sn):
         sn.sn_build_ts(basis, tok, workspace=torch.empty(16, dtype=torch.uint8, device="cuda"))
     assert e.value.status == sn.SN_ERR_INVALID_ARG
     basis.destroy()
+
+
+@pytest.mark.parametrize("k", [1, 15, 16, 17, 41, 64, 127, 128])
+@pytest.mark.parametrize("positions", ["implicit", "explicit", "none"])
+def test_projected_whole_tiles(sn, oracle, k, positions):
+    """d = 512 is too short for a tile's d-range to be split, so every tile's
+    epilogue subtracts its rows of TU and PU itself: all widths, a ragged last
+    tile, and an invalid id and position."""
+    T, n, d, vocab = 300, 70, 512, 200
+    inp = inputs(T, n, d, k, vocab, seed=k)
+    rng = np.random.default_rng(k)
+    ids, pos = inp["ids"].copy(), None
+    ids[131] = vocab
+    if positions == "explicit":
+        pos = rng.integers(0, n, T).astype(np.int32)
+        pos[7] = n
+    pe = None if positions == "none" else inp["pos_emb"]
+    basis = sn.Basis(dev(inp["U"]))
+    TU, PU = sn.sn_project_tables(basis, dev(inp["tok_emb"]), pos_emb=None if pe is None else dev(pe))
+    C = sn.sn_compress_fwd_projected(basis, dev(inp["X"]), dev(ids), TU, n, PU=PU,
+                                     pos=None if pos is None else dev(pos))
+    with pytest.raises(sn.SNError) as e:
+        sn.sn_check_errors(basis)
+    assert e.value.status == sn.SN_ERR_BAD_ID
+    _, C64, _ = oracle.compress_fwd(inp["X"], ids, inp["tok_emb"], inp["U"], n, pos_emb=pe, pos=pos)
+    assert_parity(host(C), C64, "bf16")
+    basis.destroy()
