@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(kCols) k_adamw_moments(const GT *__restrict__ 
                                                           int64_t cols, float b1, float b2,
                                                           float vcorr, float *__restrict__ colsum)
 {
+    griddep_wait();
     const int64_t c = (int64_t)blockIdx.x * kCols + threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.y * kRows;
     if (c >= cols)
@@ -65,6 +66,7 @@ __global__ void __launch_bounds__(kCols) k_adamw_apply(float *__restrict__ W,
                                                         float eps, float lam, float inv_rows,
                                                         const float *__restrict__ colsum)
 {
+    griddep_wait();
     const int64_t c = (int64_t)blockIdx.x * kCols + threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.y * kRows;
     if (c >= cols)
@@ -104,6 +106,7 @@ __global__ void __launch_bounds__(kCols) k_adamw_v4(const GT *__restrict__ g, fl
                                                      int64_t rows, int64_t cols, float b2, float vcorr,
                                                      float *__restrict__ colsum)
 {
+    griddep_wait();
     const int64_t c = 4 * ((int64_t)blockIdx.x * kCols + threadIdx.x);
     const int64_t r0 = (int64_t)blockIdx.y * kRowsV;
     if (c >= cols)
@@ -146,6 +149,7 @@ __global__ void __launch_bounds__(kCols) k_adamw_mw4(const GT *__restrict__ g, f
                                                       float eps, float lam, float inv_rows,
                                                       const float *__restrict__ colsum)
 {
+    griddep_wait();
     const int64_t c = 4 * ((int64_t)blockIdx.x * kCols + threadIdx.x);
     const int64_t r0 = (int64_t)blockIdx.y * kRowsV;
     if (c >= cols)

@@ -480,6 +480,7 @@ __global__ void __launch_bounds__(256, 4) k_residual(const __nv_bfloat16 *__rest
                                                      const __nv_bfloat16 *__restrict__ Cg, int64_t nc,
                                                      double *acc)
 {
+    griddep_wait();
     double s = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -546,9 +547,10 @@ cudaError_t grassmann_residual(const sn_basis &b, const __nv_bfloat16 *G,
 {
     const int64_t want = (T * b.d / 8 + 255) / 256;
     const int grid = (int)std::min<int64_t>(std::max<int64_t>(want, 1), 4 * sm_count());
-    k_residual<<<grid, 256, 0, s>>>(G, T * b.d, Cg, T * b.k, acc);
+    const cudaError_t e =
+        launch_dependent(k_residual, dim3(grid), dim3(256), 0, s, G, T * b.d, Cg, T * b.k, acc);
     count_launch();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // workspace: Y, G1, G2 and the barrier (k x k fp32 each, two spare ones) | A, Q1

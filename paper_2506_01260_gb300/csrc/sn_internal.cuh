@@ -46,6 +46,63 @@ namespace sn {
 // Counts every kernel the library launches (reported by sn_launch_count).
 void count_launch(int n = 1);
 
+// ---- dependent launches ----------------------------------------------------------
+// A kernel launched with programmatic stream serialization may be set up before the
+// previous kernel of its stream has ended: griddep_wait blocks until that one has
+// completed and its writes are visible (a no-op after a normal launch or any
+// other kind of predecessor).  The library's kernels call it before their first
+// access to global memory, so a launch overlaps the end of whatever ran before it, and
+// none completes before its predecessor has.
+//
+// griddep_launch_dependents lets the next such kernel start as soon as every CTA of
+// this one has called it, instead of when they end.  Only grids of at most kFewCtas
+// call it: their successor finds idle SMs.  Called by every kernel, the
+// successor's first CTAs crowd onto the SMs that happen to be free, and the four
+// boundary calls took 76 us instead of 67 (1B class, 128 CTAs a grid), 192 instead of
+// 182 (8B class), in fp32 153 instead of 137.
+constexpr unsigned kFewCtas = 64;
+
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch_dependents()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void griddep_start()
+{
+    if (gridDim.x <= kFewCtas)
+        griddep_launch_dependents();
+    griddep_wait();
+}
+
+// Launch `kernel` in clusters of `cluster` CTAs along x, as a dependent of the
+// previous kernel of the stream.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_clusters(void (*kernel)(KArgs...), int cluster, dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t s, const Args &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                             cudaStream_t s, const Args &...args)
+{
+    return launch_clusters(kernel, 1, grid, block, smem, s, args...);
+}
+
 // ---- CUDA-core kernels (fp32 path) -------------------------------------------
 cudaError_t simt_compress(const sn_basis &b, const float *X, const int32_t *ids, const int32_t *pos,
                           int64_t T, int seq_len, const float *tok, int64_t vocab, const float *pe,

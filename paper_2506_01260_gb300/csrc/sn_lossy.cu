@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(kThreads) k_topk(const uint16_t *__restrict__ 
                                                     int d, int kk, uint16_t *__restrict__ vals,
                                                     uint16_t *__restrict__ cols)
 {
+    griddep_wait();
     extern __shared__ __align__(16) uint8_t tk_smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nch = d / 8, per_lane = (nch + 31) / 32;
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(kThreads) k_topk_restore(const uint16_t *__res
                                                             int64_t T, int d, int kk,
                                                             uint16_t *__restrict__ out)
 {
+    griddep_wait();
     for (int64_t t = blockIdx.x; t < T; t += gridDim.x) {
         uint16_t *dst = out + t * (int64_t)d;
         __syncthreads();
@@ -324,6 +326,7 @@ __global__ void __launch_bounds__(kThreads) k_sign(const uint16_t *__restrict__ 
                                                     uint32_t *__restrict__ bits,
                                                     float *__restrict__ scale)
 {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
     const int nch = d / 8, words = (d + 31) / 32;
@@ -376,6 +379,7 @@ __global__ void __launch_bounds__(kThreads) k_sign_restore(const uint32_t *__res
                                                             int64_t T, int d,
                                                             uint16_t *__restrict__ out)
 {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
     const int nch = d / 8, words = (d + 31) / 32;
@@ -436,6 +440,7 @@ __global__ void __launch_bounds__(kThreads) k_quant(const uint16_t *__restrict__
                                                      uint8_t *__restrict__ codes,
                                                      float *__restrict__ scale)
 {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
     const int nch = d / 8;
@@ -512,6 +517,7 @@ __global__ void __launch_bounds__(kThreads) k_quant_restore(const uint8_t *__res
                                                              int64_t T, int d,
                                                              uint16_t *__restrict__ out)
 {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = ((int64_t)gridDim.x * kThreads) >> 5;
     const int nch = d / 8;
@@ -548,6 +554,14 @@ int warp_grid(int64_t T)
     return (int)(need < 8 * (int64_t)sms ? need : 8 * (int64_t)sms);
 }
 
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kernel)(KArgs...), int grid, size_t smem, cudaStream_t s, const Args &...args)
+{
+    const cudaError_t e = launch_dependent(kernel, dim3(grid), dim3(kThreads), smem, s, args...);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int M>
 cudaError_t launch_topk(const void *X, int64_t T, int d, int kk, void *vals, uint16_t *cols,
                         cudaStream_t s)
@@ -565,10 +579,8 @@ cudaError_t launch_topk(const void *X, int64_t T, int d, int kk, void *vals, uin
         return e;
     const int64_t resident = (int64_t)sms * (per_sm > 0 ? per_sm : 1);   // one wave
     const int64_t need = (T + kWarps - 1) / kWarps;
-    k_topk<M><<<(int)(need < resident ? need : resident), kThreads, smem, s>>>(
-        (const uint16_t *)X, T, d, kk, (uint16_t *)vals, cols);
-    count_launch();
-    return cudaGetLastError();
+    return launch(k_topk<M>, (int)(need < resident ? need : resident), smem, s, (const uint16_t *)X, T, d,
+                  kk, (uint16_t *)vals, cols);
 }
 
 }  // namespace
@@ -591,18 +603,14 @@ cudaError_t lossy_topk(const void *X, int64_t T, int d, int kk, void *vals, uint
 cudaError_t lossy_topk_restore(const void *vals, const uint16_t *cols, int64_t T, int d, int kk,
                                void *out, cudaStream_t s)
 {
-    k_topk_restore<<<row_grid(T), kThreads, 0, s>>>((const uint16_t *)vals, cols, T, d, kk,
-                                                     (uint16_t *)out);
-    count_launch();
-    return cudaGetLastError();
+    return launch(k_topk_restore, row_grid(T), 0, s, (const uint16_t *)vals, cols, T, d, kk,
+                  (uint16_t *)out);
 }
 
 cudaError_t lossy_sign(const void *X, int64_t T, int d, uint32_t *bits, float *scale,
                        cudaStream_t s)
 {
-    k_sign<<<warp_grid(T), kThreads, 0, s>>>((const uint16_t *)X, T, d, bits, scale);
-    count_launch();
-    return cudaGetLastError();
+    return launch(k_sign, warp_grid(T), 0, s, (const uint16_t *)X, T, d, bits, scale);
 }
 
 // The 8-bit quantizer reads every row twice; the second read hits L2 only if
@@ -624,33 +632,21 @@ cudaError_t lossy_quant(const void *X, int64_t T, int d, int format, uint8_t *co
                         cudaStream_t s)
 {
     const int grid = quant_grid(T, d);
-    if (format == SN_Q_INT8)
-        k_quant<SN_Q_INT8><<<grid, kThreads, 0, s>>>((const uint16_t *)X, T, d, codes, scale);
-    else
-        k_quant<SN_Q_E4M3><<<grid, kThreads, 0, s>>>((const uint16_t *)X, T, d, codes, scale);
-    count_launch();
-    return cudaGetLastError();
+    return launch(format == SN_Q_INT8 ? k_quant<SN_Q_INT8> : k_quant<SN_Q_E4M3>, grid, 0, s,
+                  (const uint16_t *)X, T, d, codes, scale);
 }
 
 cudaError_t lossy_quant_restore(const uint8_t *codes, const float *scale, int64_t T, int d,
                                 int format, void *out, cudaStream_t s)
 {
-    if (format == SN_Q_INT8)
-        k_quant_restore<SN_Q_INT8><<<warp_grid(T), kThreads, 0, s>>>(codes, scale, T, d,
-                                                                     (uint16_t *)out);
-    else
-        k_quant_restore<SN_Q_E4M3><<<warp_grid(T), kThreads, 0, s>>>(codes, scale, T, d,
-                                                                     (uint16_t *)out);
-    count_launch();
-    return cudaGetLastError();
+    return launch(format == SN_Q_INT8 ? k_quant_restore<SN_Q_INT8> : k_quant_restore<SN_Q_E4M3>,
+                  warp_grid(T), 0, s, codes, scale, T, d, (uint16_t *)out);
 }
 
 cudaError_t lossy_sign_restore(const uint32_t *bits, const float *scale, int64_t T, int d,
                                void *out, cudaStream_t s)
 {
-    k_sign_restore<<<warp_grid(T), kThreads, 0, s>>>(bits, scale, T, d, (uint16_t *)out);
-    count_launch();
-    return cudaGetLastError();
+    return launch(k_sign_restore, warp_grid(T), 0, s, bits, scale, T, d, (uint16_t *)out);
 }
 
 }  // namespace sn

@@ -101,30 +101,6 @@ __device__ __forceinline__ float ld_cluster(uint32_t a, uint32_t rank)
     return v;
 }
 
-// Launch a kernel in clusters of `cluster` CTAs along x.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_clusters(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem,
-                            int cluster, cudaStream_t s, Args... args)
-{
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess)
-        return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // CTAs per cluster that share one output tile's reduction: the power of two up
 // to 8 with the least (rounds of the grid) x (steps per CTA + 3 for its start + one
 // for each CTA whose partial sums meet), every CTA keeping at least one step.  Among
@@ -196,6 +172,7 @@ __global__ void __launch_bounds__(CTHREADS) k_simt_compress(const SimtCompress p
     const int rank = (int)(blockIdx.x % p.split);
     const int64_t t0 = (int64_t)(blockIdx.x / p.split) * CTOK;
     const bool has_pe = GATHER && p.pe != nullptr;
+    griddep_wait();
     if (tid < CTOK)
         rstate[tid] = token_rows(t0 + tid, p.T, GATHER, p.ids, p.pos, p.seq_len, p.vocab, has_pe,
                                  p.d, &rtok[tid], &rpe[tid], p.err);
@@ -388,6 +365,7 @@ __global__ void __launch_bounds__(ETHREADS, 2) k_simt_expand(const SimtExpand p)
     __shared__ int rstate[2 * ETILE];
     const int64_t c0 = (int64_t)blockIdx.x * ETILE;
     const bool has_pe = EMB && p.pe != nullptr;
+    griddep_wait();
     if (p.ldr % 4 == 0) {
         for (int e = tid; e < p.k * (ETILE / 4); e += ETHREADS) {
             const int j = e / (ETILE / 4), q = 4 * (e % (ETILE / 4));
@@ -597,6 +575,7 @@ __global__ void __launch_bounds__(PTHREADS) k_simt_project_a(const SimtProject p
         acc[j][0] = acc[j][1] = 0ull;
     const int stride = BROWS * p.split;
     int row = rank * BROWS;
+    griddep_wait();
     load_w(row + PROWS * group);
     load_u(row, 0);
     for (int it = 0; row < p.d; ++it, row += stride) {
@@ -717,9 +696,11 @@ cudaError_t launch_compress_f32(SimtCompress p, bool gather, int sms, cudaStream
     // registers let two (gather) or three CTAs share an SM
     p.split = cluster_split(tiles, steps, (int64_t)sms * (gather ? 2 : 3));
     const unsigned grid = (unsigned)(tiles * p.split);
-    const cudaError_t e =
-        gather ? launch_clusters(k_simt_compress<WN, TN, true>, grid, CTHREADS, smem, p.split, s, p)
-               : launch_clusters(k_simt_compress<WN, TN, false>, grid, CTHREADS, smem, p.split, s, p);
+    void (*const kernel)(SimtCompress) =
+        gather ? k_simt_compress<WN, TN, true> : k_simt_compress<WN, TN, false>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = launch_clusters(kernel, p.split, dim3(grid), dim3(CTHREADS), smem, s, p);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -745,9 +726,10 @@ cudaError_t launch_expand_f32(const SimtExpand &p, int sms, cudaStream_t s)
             gy = y;
         }
     }
-    k_simt_expand<EMB><<<dim3((unsigned)ctiles, (unsigned)gy), ETHREADS, smem, s>>>(p);
+    e = launch_dependent(k_simt_expand<EMB>, dim3((unsigned)ctiles, (unsigned)gy), dim3(ETHREADS), smem,
+                         s, p);
     count_launch();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int WN, int JT>
@@ -758,8 +740,12 @@ cudaError_t launch_project_a(SimtProject p, int sms, cudaStream_t s)
     const int64_t tiles = (p.cols + 127) / 128;
     const int steps = (p.d + PROWS * G - 1) / (PROWS * G);
     p.split = cluster_split(tiles, steps, sms);
-    const cudaError_t e = launch_clusters(k_simt_project_a<WN, JT>, (unsigned)(tiles * p.split),
-                                          PTHREADS, stage > red ? stage : red, p.split, s, p);
+    constexpr size_t smem = stage > red ? stage : red;
+    cudaError_t e = cudaFuncSetAttribute(k_simt_project_a<WN, JT>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+        e = launch_clusters(k_simt_project_a<WN, JT>, p.split, dim3((unsigned)(tiles * p.split)),
+                            dim3(PTHREADS), smem, s, p);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    griddep_wait();   // the projection's third pass: the previous passes' writes are visible
+    griddep_start();               // the previous kernel's writes are visible
     const int nitems = p.ntiles * p.chunks;
 
     if (warp == 0) {
@@ -306,37 +306,14 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
 
 }  // namespace
 
-cudaError_t launch_expand(int amode, const ExpandParams &p, int grid, cudaStream_t s,
-                          bool dependent)
+cudaError_t launch_expand(int amode, const ExpandParams &p, int grid, cudaStream_t s)
 {
     const ExpandPlan pl = expand_plan(p.katoms, p.stages);
-    cudaError_t e;
-    if (amode == AMODE_REPACK) {
-        e = cudaFuncSetAttribute(k_expand<AMODE_REPACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 pl.total);
-        if (e == cudaSuccess)
-            k_expand<AMODE_REPACK><<<grid, kExpandThreads, pl.total, s>>>(p);
-    } else {
-        e = cudaFuncSetAttribute(k_expand<AMODE_TMA>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 pl.total);
-        if (e == cudaSuccess && dependent) {
-            // may start while the previous kernel of the stream finishes (it
-            // waits for it in griddep_wait before touching global memory)
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(grid);
-            cfg.blockDim = dim3(kExpandThreads);
-            cfg.dynamicSmemBytes = pl.total;
-            cfg.stream = s;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            e = cudaLaunchKernelEx(&cfg, k_expand<AMODE_TMA>, p);
-        } else if (e == cudaSuccess) {
-            k_expand<AMODE_TMA><<<grid, kExpandThreads, pl.total, s>>>(p);
-        }
-    }
+    void (*const kernel)(ExpandParams) = amode == AMODE_REPACK ? k_expand<AMODE_REPACK> : k_expand<AMODE_TMA>;
+    cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.total);
+    if (e == cudaSuccess)
+        e = launch_dependent(kernel, dim3(grid), dim3(kExpandThreads), pl.total, s, p);
     if (e != cudaSuccess)
         return e;
     count_launch();

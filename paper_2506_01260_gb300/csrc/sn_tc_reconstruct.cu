@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    griddep_start();               // the previous kernel's writes are visible
     const int nitems = p.ntiles * p.chunks;
 
     if (warp == 0) {
@@ -613,6 +614,7 @@ __global__ void __launch_bounds__(kReconThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    griddep_start();
     const int nitems = p.ntiles * p.chunks;    // p.ntiles counts tile pairs here
 
     if (warp == 0) {
@@ -968,9 +970,10 @@ cudaError_t launch_reconstruct(const ExpandParams &p, int grid, cudaStream_t s)
     const ReconPlan pl = recon_plan(p.katoms, p.has_pe, p.stages, p.estages);
     cudaError_t e = cudaFuncSetAttribute(k_reconstruct, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          pl.total);
+    if (e == cudaSuccess)
+        e = launch_dependent(k_reconstruct, dim3(grid), dim3(kReconThreads), pl.total, s, p);
     if (e != cudaSuccess)
         return e;
-    k_reconstruct<<<grid, kReconThreads, pl.total, s>>>(p);
     count_launch();
     return cudaGetLastError();
 }
@@ -980,9 +983,10 @@ cudaError_t launch_reconstruct_pair(const ExpandParams &p, int grid, cudaStream_
     const PairPlan pl = pair_plan(p.katoms, p.stages, p.estages);
     cudaError_t e = cudaFuncSetAttribute(k_reconstruct_pair, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          pl.total);
+    if (e == cudaSuccess)
+        e = launch_dependent(k_reconstruct_pair, dim3(grid), dim3(kReconThreads), pl.total, s, p);
     if (e != cudaSuccess)
         return e;
-    k_reconstruct_pair<<<grid, kReconThreads, pl.total, s>>>(p);
     count_launch();
     return cudaGetLastError();
 }
