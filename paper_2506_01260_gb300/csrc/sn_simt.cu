@@ -82,6 +82,17 @@ __device__ __forceinline__ void cp_async_4(uint32_t dst, const void *src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
+// `bytes` (0 to 16) of the 16, the rest zeros
+__device__ __forceinline__ void cp_async_part(uint32_t dst, const void *src, unsigned bytes)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -104,9 +115,10 @@ __device__ __forceinline__ float ld_cluster(uint32_t a, uint32_t rank)
 // CTAs per cluster that share one output tile's reduction: the power of two up
 // to 8 with the least (rounds of the grid) x (steps per CTA + 3 for its start + one
 // for each CTA whose partial sums meet), every CTA keeping at least one step.  Among
-// equal costs, the fewest CTAs.  Measured, with 1 / 2 / 4 / 8 CTAs: projection of
-// [2048, 2048] at k = 20 (16 tiles) 74 / 48 / 33 / 37 us, of [2048, 8192] (64 tiles)
-// 92 / 67 / 72 / 90 us; compress of 8192 x 2048 (256 tiles) 31 / 34 / 35 / 43 us.
+// equal costs, the fewest CTAs.  Measured on whole calls, with 1 / 2 / 4 / 8 CTAs (W one
+// step ahead): projection of [2048, 2048] at k = 20 (16 tiles) 74 / 48 / 33 / 37 us, of
+// [2048, 8192] (64 tiles) 92 / 67 / 72 / 90 us; compress of 8192 x 2048 (256 tiles) 31 /
+// 34 / 35 / 43 us.
 int cluster_split(int64_t tiles, int steps, int64_t slots)
 {
     int best = 1;
@@ -520,14 +532,17 @@ __global__ void __launch_bounds__(ETHREADS, 2) k_simt_expand(const SimtExpand p)
 // ---- A = U^T W (fp32 [k, cols]), the projection's first pass ---------------------
 // A warp owns 128 columns of W (a thread four, as two pairs) and JT columns of U;
 // WN warps form a group that covers all k, and the groups of a CTA and the CTAs of
-// a cluster take blocks of eight rows of W in turn.  W goes from HBM straight to
-// registers (eight 512-byte rows a warp, a block ahead); U comes a block ahead by
-// cp.async from the paired copy u32p and is read by broadcast, two rows x two
-// columns a load for 8 packed FMAs.  [2048, 2048] and [2048, 8192] at k = 20: 20 and
-// 36 us, where one thread per column walked all of d with one load of U per FMA, on
-// 16 and 64 CTAs, 1297 and 1339 us.
+// a cluster take blocks of eight rows of W in turn.  W and U (paired copy u32p) come
+// through a ring of four steps by cp.async: a thread copies and reads its own
+// 16-byte pieces of W, U is shared and read by broadcast, two rows x two columns a
+// load for 8 packed FMAs.  [2048, 2048] and [2048, 8192] at k = 20: 18 and 29 us (HBM
+// 2.5 and 10, FMA pipe 2.3 and 9 on all SMs), 20 and 35 with W a single step ahead in
+// registers, and 1297 and 1339 with a thread per column that walked all of d with one
+// load of U per FMA.  The FMA pipe is 42% busy: two warps a scheduler issue 0.4 a
+// cycle.  Three CTAs of four warps on an SM were slower (18 and 33 us).
 constexpr int PROWS = 8;        // rows of W per group and step
 constexpr int PTHREADS = 256;
+constexpr int PSTEPS = 4;       // steps in the ring
 
 struct SimtProject {
     const float *up, *W;
@@ -541,77 +556,74 @@ __global__ void __launch_bounds__(PTHREADS) k_simt_project_a(const SimtProject p
 {
     constexpr int G = PTHREADS / 32 / WN, KP = WN * JT;
     constexpr int BROWS = PROWS * G;                // rows of W per CTA and step
-    extern __shared__ __align__(16) float smp[];    // U: [2][BROWS / 2][KP][2]
+    extern __shared__ __align__(16) float smp[];    // U [PSTEPS][BROWS / 2][KP][2], then W
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int group = warp / WN, jg = warp % WN;
     const int rank = (int)(blockIdx.x % p.split);
     const int64_t c0 = (int64_t)(blockIdx.x / p.split) * 128, c = c0 + 4 * lane;
+    float *ws = smp + PSTEPS * BROWS * KP + 4 * tid;    // [PSTEPS][PROWS][PTHREADS][4]
 
-    ulonglong2 w[PROWS];
-    auto load_w = [&](int row0) {
-        const float *src = p.W + (int64_t)row0 * p.ld + c;
+    // this thread's 16 bytes of a row of W, zero-filled past the last column
+    const unsigned wbytes = (unsigned)(4 * max((int64_t)0, min((int64_t)4, p.cols - c)));
+    const float *wsrc = p.W + (wbytes ? c : 0);
+    const int stride = BROWS * p.split;
+    auto fetch = [&](int step) {
+        const int row0 = rank * BROWS + step * stride, b = step % PSTEPS;
+        if (row0 < p.d) {
+            const int r = row0 + PROWS * group;
+            if (r < p.d)                            // d is a multiple of 8: all rows or none
 #pragma unroll
-        for (int i = 0; i < PROWS; ++i, src += p.ld) {
-            w[i] = make_ulonglong2(0ull, 0ull);
-            if (row0 < p.d) {                       // d is a multiple of 8: all rows or none
-                if (c + 4 <= p.cols)
-                    w[i] = __ldg((const ulonglong2 *)src);
-                else if (c < p.cols)
-                    w[i] = make_ulonglong2(pack2(src[0], c + 1 < p.cols ? src[1] : 0.f),
-                                           pack2(c + 2 < p.cols ? src[2] : 0.f, 0.f));
-            }
+                for (int i = 0; i < PROWS; ++i)
+                    cp_async_part(smem_addr(ws + (b * PROWS + i) * 4 * PTHREADS),
+                                  wsrc + (int64_t)(r + i) * p.ld, wbytes);
+            // u32p is padded to 32 rows past d
+            const int n = min(BROWS, (p.d + 31) / 32 * 32 - row0) * KP / 4;
+            const float *src = p.up + (int64_t)row0 * KP;
+            const uint32_t dst = smem_addr(smp + b * BROWS * KP);
+            for (int f = tid; f < n; f += PTHREADS)
+                cp_async_16(dst + 16 * f, src + 4 * f);
         }
-    };
-    auto load_u = [&](int row0, int b) {            // u32p is padded to 32 rows past d
-        const int n = min(BROWS, (p.d + 31) / 32 * 32 - row0) * KP / 4;
-        const float *src = p.up + (int64_t)row0 * KP;
-        const uint32_t dst = smem_addr(smp + b * BROWS * KP);
-        for (int f = tid; f < n; f += PTHREADS)
-            cp_async_16(dst + 16 * f, src + 4 * f);
+        cp_async_commit();
     };
     f32x2 acc[JT][2];
 #pragma unroll
     for (int j = 0; j < JT; ++j)
         acc[j][0] = acc[j][1] = 0ull;
-    const int stride = BROWS * p.split;
-    int row = rank * BROWS;
     griddep_wait();
-    load_w(row + PROWS * group);
-    load_u(row, 0);
-    for (int it = 0; row < p.d; ++it, row += stride) {
-        const int b = it & 1;
-        cp_async_wait_all();
-        __syncthreads();                            // this step's U is staged, the last one's used up
-        ulonglong2 cur[PROWS];
 #pragma unroll
-        for (int i = 0; i < PROWS; ++i)
-            cur[i] = w[i];
-        if (row + stride < p.d) {
-            load_w(row + stride + PROWS * group);
-            load_u(row + stride, b ^ 1);
-        }
-        if (row + PROWS * group >= p.d)             // past the end: no rows of U are staged
+    for (int s = 0; s < PSTEPS - 1; ++s)
+        fetch(s);
+    for (int it = 0, row = rank * BROWS; row < p.d; ++it, row += stride) {
+        const int b = it % PSTEPS;
+        cp_async_wait<PSTEPS - 2>();
+        __syncthreads();                            // this step has landed, the last one is used up
+        fetch(it + PSTEPS - 1);
+        if (row + PROWS * group >= p.d)             // past the end: no rows were fetched
             continue;
         const float *ut = smp + b * BROWS * KP + PROWS * group * KP + 2 * jg * JT;
+        const float *wt = ws + b * PROWS * 4 * PTHREADS;
 #pragma unroll
         for (int i = 0; i < PROWS / 2; ++i) {
+            const ulonglong2 w0 = *(const ulonglong2 *)(wt + 2 * i * 4 * PTHREADS);
+            const ulonglong2 w1 = *(const ulonglong2 *)(wt + (2 * i + 1) * 4 * PTHREADS);
 #pragma unroll
             for (int j = 0; j < JT; j += 2) {
                 // (U[2i, j], U[2i + 1, j], U[2i, j + 1], U[2i + 1, j + 1])
                 const float4 u = *(const float4 *)(ut + 2 * i * KP + 2 * j);
                 const f32x2 a0 = pack2(u.x, u.x), a1 = pack2(u.y, u.y);
                 const f32x2 b0 = pack2(u.z, u.z), b1 = pack2(u.w, u.w);
-                acc[j][0] = fma2(a0, cur[2 * i].x, acc[j][0]);
-                acc[j][1] = fma2(a0, cur[2 * i].y, acc[j][1]);
-                acc[j + 1][0] = fma2(b0, cur[2 * i].x, acc[j + 1][0]);
-                acc[j + 1][1] = fma2(b0, cur[2 * i].y, acc[j + 1][1]);
-                acc[j][0] = fma2(a1, cur[2 * i + 1].x, acc[j][0]);
-                acc[j][1] = fma2(a1, cur[2 * i + 1].y, acc[j][1]);
-                acc[j + 1][0] = fma2(b1, cur[2 * i + 1].x, acc[j + 1][0]);
-                acc[j + 1][1] = fma2(b1, cur[2 * i + 1].y, acc[j + 1][1]);
+                acc[j][0] = fma2(a0, w0.x, acc[j][0]);
+                acc[j][1] = fma2(a0, w0.y, acc[j][1]);
+                acc[j + 1][0] = fma2(b0, w0.x, acc[j + 1][0]);
+                acc[j + 1][1] = fma2(b0, w0.y, acc[j + 1][1]);
+                acc[j][0] = fma2(a1, w1.x, acc[j][0]);
+                acc[j][1] = fma2(a1, w1.y, acc[j][1]);
+                acc[j + 1][0] = fma2(b1, w1.x, acc[j + 1][0]);
+                acc[j + 1][1] = fma2(b1, w1.y, acc[j + 1][1]);
             }
         }
     }
+    cp_async_wait_all();                            // (empty groups only)
     // partial sums [G][KP][128] of the groups, then of the cluster's CTAs
     float *red = smp;
     __syncthreads();
@@ -736,7 +748,8 @@ template <int WN, int JT>
 cudaError_t launch_project_a(SimtProject p, int sms, cudaStream_t s)
 {
     constexpr int G = PTHREADS / 32 / WN, KP = WN * JT;
-    constexpr size_t stage = sizeof(float) * 2 * PROWS * G * KP, red = sizeof(float) * G * KP * 128;
+    constexpr size_t stage = sizeof(float) * PSTEPS * (PROWS * G * KP + PROWS * 4 * PTHREADS);
+    constexpr size_t red = sizeof(float) * G * KP * 128;
     const int64_t tiles = (p.cols + 127) / 128;
     const int steps = (p.d + PROWS * G - 1) / (PROWS * G);
     p.split = cluster_split(tiles, steps, sms);
