@@ -13,6 +13,8 @@
 // adjacent columns (16-byte accesses, rows unrolled by four) of a block of rows
 // when the column count is a multiple of 4, else one column; every access is
 // coalesced along the columns.
+#include <algorithm>
+
 #include "sn_internal.cuh"
 
 namespace sn {
@@ -20,6 +22,13 @@ namespace {
 
 constexpr int kCols = 256;   // columns per block (one per thread)
 constexpr int kRows = 64;    // rows per block
+
+__global__ void __launch_bounds__(kCols) k_zero(float *__restrict__ p, int64_t n)
+{
+    griddep_wait();
+    for (int64_t i = (int64_t)blockIdx.x * kCols + threadIdx.x; i < n; i += (int64_t)gridDim.x * kCols)
+        p[i] = 0.f;
+}
 
 template <typename GT>
 __device__ __forceinline__ float load_grad(const GT *g, int64_t e);
@@ -195,7 +204,9 @@ cudaError_t adamw_rowconst(bool grad_bf16, float *W, const void *g, float *M, fl
                            int64_t rows, int64_t cols, int64_t t, float lr, float b1, float b2,
                            float eps, float lam, float *colsum, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(colsum, 0, sizeof(float) * (size_t)cols, s);
+    // three dependent launches: a memset between two kernels would end the overlap
+    cudaError_t e = launch_dependent(k_zero, dim3((unsigned)std::min<int64_t>((cols + kCols - 1) / kCols, 152)),
+                                     dim3(kCols), 0, s, colsum, cols);
     if (e != cudaSuccess)
         return e;
     // bias corrections of step t, in double before rounding to fp32
@@ -206,31 +217,35 @@ cudaError_t adamw_rowconst(bool grad_bf16, float *W, const void *g, float *M, fl
                         (unsigned)((rows + kRowsV - 1) / kRowsV));
         const float inv_rows = (float)(1.0 / (double)rows);
         if (grad_bf16) {
-            k_adamw_v4<__nv_bfloat16><<<grid, kCols, 0, s>>>((const __nv_bfloat16 *)g, V, rows,
-                                                             cols, b2, vcorr, colsum);
-            k_adamw_mw4<__nv_bfloat16><<<grid, kCols, 0, s>>>((const __nv_bfloat16 *)g, W, M, rows,
-                                                              cols, b1, lr, mcorr, eps, lam,
-                                                              inv_rows, colsum);
+            const __nv_bfloat16 *gp = (const __nv_bfloat16 *)g;
+            e = launch_dependent(k_adamw_v4<__nv_bfloat16>, grid, dim3(kCols), 0, s, gp, V, rows, cols, b2,
+                                 vcorr, colsum);
+            if (e == cudaSuccess)
+                e = launch_dependent(k_adamw_mw4<__nv_bfloat16>, grid, dim3(kCols), 0, s, gp, W, M, rows,
+                                     cols, b1, lr, mcorr, eps, lam, inv_rows, colsum);
         } else {
-            k_adamw_v4<float><<<grid, kCols, 0, s>>>((const float *)g, V, rows, cols, b2, vcorr,
-                                                     colsum);
-            k_adamw_mw4<float><<<grid, kCols, 0, s>>>((const float *)g, W, M, rows, cols, b1, lr,
-                                                      mcorr, eps, lam, inv_rows, colsum);
+            const float *gp = (const float *)g;
+            e = launch_dependent(k_adamw_v4<float>, grid, dim3(kCols), 0, s, gp, V, rows, cols, b2, vcorr,
+                                 colsum);
+            if (e == cudaSuccess)
+                e = launch_dependent(k_adamw_mw4<float>, grid, dim3(kCols), 0, s, gp, W, M, rows, cols, b1,
+                                     lr, mcorr, eps, lam, inv_rows, colsum);
         }
-        count_launch(2);
-        return cudaGetLastError();
+        count_launch(3);
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
     const dim3 grid((unsigned)((cols + kCols - 1) / kCols), (unsigned)((rows + kRows - 1) / kRows));
     if (grad_bf16)
-        k_adamw_moments<__nv_bfloat16><<<grid, kCols, 0, s>>>(
-            (const __nv_bfloat16 *)g, M, V, rows, cols, b1, b2, vcorr, colsum);
+        e = launch_dependent(k_adamw_moments<__nv_bfloat16>, grid, dim3(kCols), 0, s,
+                             (const __nv_bfloat16 *)g, M, V, rows, cols, b1, b2, vcorr, colsum);
     else
-        k_adamw_moments<float><<<grid, kCols, 0, s>>>((const float *)g, M, V, rows, cols, b1, b2,
-                                                     vcorr, colsum);
-    k_adamw_apply<<<grid, kCols, 0, s>>>(W, M, rows, cols, lr, mcorr, eps, lam,
-                                         (float)(1.0 / (double)rows), colsum);
-    count_launch(2);
-    return cudaGetLastError();
+        e = launch_dependent(k_adamw_moments<float>, grid, dim3(kCols), 0, s, (const float *)g, M, V, rows,
+                             cols, b1, b2, vcorr, colsum);
+    if (e == cudaSuccess)
+        e = launch_dependent(k_adamw_apply, grid, dim3(kCols), 0, s, W, M, rows, cols, lr, mcorr, eps, lam,
+                             (float)(1.0 / (double)rows), colsum);
+    count_launch(3);
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace sn

@@ -74,6 +74,30 @@ __device__ __forceinline__ void griddep_start()
     griddep_wait();
 }
 
+// ---- clusters ----------------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    cluster_arrive();
+    cluster_wait();
+}
+// the fp32 at shared address `a` of the cluster's CTA `rank`
+__device__ __forceinline__ float ld_cluster(uint32_t a, uint32_t rank)
+{
+    uint32_t r;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
+    return v;
+}
+
 // Launch `kernel` in clusters of `cluster` CTAs along x, as a dependent of the
 // previous kernel of the stream.
 template <typename... KArgs, typename... Args>

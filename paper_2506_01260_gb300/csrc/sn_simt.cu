@@ -97,21 +97,6 @@ __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// the fp32 at shared address `a` of the cluster's CTA `rank`
-__device__ __forceinline__ float ld_cluster(uint32_t a, uint32_t rank)
-{
-    uint32_t r;
-    float v;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
-    return v;
-}
-
 // CTAs per cluster that share one output tile's reduction: the power of two up
 // to 8 with the least (rounds of the grid) x (steps per CTA + 3 for its start + one
 // for each CTA whose partial sums meet), every CTA keeping at least one step.  Among
