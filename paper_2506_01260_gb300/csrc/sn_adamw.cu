@@ -21,7 +21,7 @@ namespace sn {
 namespace {
 
 constexpr int kCols = 256;   // columns per block (one per thread)
-constexpr int kRows = 64;    // rows per block
+constexpr int kRows = 16;    // rows per block
 
 __global__ void __launch_bounds__(kCols) k_zero(float *__restrict__ p, int64_t n)
 {
@@ -107,8 +107,16 @@ __device__ __forceinline__ float4 load_grad4<__nv_bfloat16>(const __nv_bfloat16 
                        __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
 }
 
-constexpr int kRowsV = 64;   // rows per block (vector kernels)
-constexpr int kUnroll = 4;
+// Rows per block and rows in flight of the two passes.  Blocks run column-major over a
+// few rows, so the GPU as a whole sweeps the arrays in order of address; the first
+// pass needs enough rows to pay for its atomics.  [4096, 14336], bf16 gradient: blocks of
+// 64 / 32 / 16 + 8 rows take 259 / 251 / 240 us (6.9 TB/s on 28 bytes an element), 8 + 8
+// rows 241, 4 + 4 rows 267; [1024, 1024]: 30 us with 64 rows (64 blocks), 13 with 16 + 8.
+// Evict-first hints on V, M and W or a reversed second pass, to find g in L2, made it
+// slower (262-271 us), and so did a single kernel of clusters that own 128 columns
+// (339), or a loop over several runs of rows in a block (263).
+constexpr int kRows1 = 16, kRows2 = 8;
+constexpr int kUnroll1 = 4, kUnroll2 = 8;
 
 template <typename GT>
 __global__ void __launch_bounds__(kCols) k_adamw_v4(const GT *__restrict__ g, float *__restrict__ V,
@@ -117,21 +125,21 @@ __global__ void __launch_bounds__(kCols) k_adamw_v4(const GT *__restrict__ g, fl
 {
     griddep_wait();
     const int64_t c = 4 * ((int64_t)blockIdx.x * kCols + threadIdx.x);
-    const int64_t r0 = (int64_t)blockIdx.y * kRowsV;
+    const int64_t r0 = (int64_t)blockIdx.y * kRows1;
     if (c >= cols)
         return;
-    const int64_t r1 = r0 + kRowsV < rows ? r0 + kRowsV : rows;
+    const int64_t r1 = r0 + kRows1 < rows ? r0 + kRows1 : rows;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t rb = r0; rb < r1; rb += kUnroll) {
-        float4 gv[kUnroll], vv[kUnroll];
+    for (int64_t rb = r0; rb < r1; rb += kUnroll1) {
+        float4 gv[kUnroll1], vv[kUnroll1];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u)
+        for (int u = 0; u < kUnroll1; ++u)
             if (rb + u < r1) {
                 gv[u] = load_grad4(g, (rb + u) * cols + c);
                 vv[u] = *(const float4 *)(V + (rb + u) * cols + c);
             }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u)
+        for (int u = 0; u < kUnroll1; ++u)
             if (rb + u < r1) {
                 float4 v;
                 v.x = b2 * vv[u].x + (1.f - b2) * gv[u].x * gv[u].x;
@@ -160,7 +168,7 @@ __global__ void __launch_bounds__(kCols) k_adamw_mw4(const GT *__restrict__ g, f
 {
     griddep_wait();
     const int64_t c = 4 * ((int64_t)blockIdx.x * kCols + threadIdx.x);
-    const int64_t r0 = (int64_t)blockIdx.y * kRowsV;
+    const int64_t r0 = (int64_t)blockIdx.y * kRows2;
     if (c >= cols)
         return;
     const float4 cs = *(const float4 *)(colsum + c);
@@ -168,11 +176,11 @@ __global__ void __launch_bounds__(kCols) k_adamw_mw4(const GT *__restrict__ g, f
                                   lr * mcorr / (sqrtf(cs.y * inv_rows) + eps),
                                   lr * mcorr / (sqrtf(cs.z * inv_rows) + eps),
                                   lr * mcorr / (sqrtf(cs.w * inv_rows) + eps));
-    const int64_t r1 = r0 + kRowsV < rows ? r0 + kRowsV : rows;
-    for (int64_t rb = r0; rb < r1; rb += kUnroll) {
-        float4 gv[kUnroll], mv[kUnroll], wv[kUnroll];
+    const int64_t r1 = r0 + kRows2 < rows ? r0 + kRows2 : rows;
+    for (int64_t rb = r0; rb < r1; rb += kUnroll2) {
+        float4 gv[kUnroll2], mv[kUnroll2], wv[kUnroll2];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u)
+        for (int u = 0; u < kUnroll2; ++u)
             if (rb + u < r1) {
                 const int64_t e = (rb + u) * cols + c;
                 gv[u] = load_grad4(g, e);
@@ -180,7 +188,7 @@ __global__ void __launch_bounds__(kCols) k_adamw_mw4(const GT *__restrict__ g, f
                 wv[u] = *(const float4 *)(W + e);
             }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u)
+        for (int u = 0; u < kUnroll2; ++u)
             if (rb + u < r1) {
                 const int64_t e = (rb + u) * cols + c;
                 float4 m, w;
@@ -198,6 +206,36 @@ __global__ void __launch_bounds__(kCols) k_adamw_mw4(const GT *__restrict__ g, f
     }
 }
 
+// The first pass over `rows` rows: V (and M, where the columns are taken singly)
+template <typename GT>
+cudaError_t moments(const GT *g, float *M, float *V, int64_t rows, int64_t cols, float b1, float b2,
+                    float vcorr, float *colsum, cudaStream_t s)
+{
+    count_launch();
+    if (cols % 4 != 0)
+        return launch_dependent(k_adamw_moments<GT>,
+                                dim3((unsigned)((cols + kCols - 1) / kCols), (unsigned)((rows + kRows - 1) / kRows)),
+                                dim3(kCols), 0, s, g, M, V, rows, cols, b1, b2, vcorr, colsum);
+    return launch_dependent(k_adamw_v4<GT>,
+                            dim3((unsigned)((cols / 4 + kCols - 1) / kCols), (unsigned)((rows + kRows1 - 1) / kRows1)),
+                            dim3(kCols), 0, s, g, V, rows, cols, b2, vcorr, colsum);
+}
+
+// The second pass: W (and M)
+template <typename GT>
+cudaError_t apply(const GT *g, float *W, float *M, int64_t rows, int64_t cols, float b1, float lr, float mcorr,
+                  float eps, float lam, float inv_rows, const float *colsum, cudaStream_t s)
+{
+    count_launch();
+    if (cols % 4 != 0)
+        return launch_dependent(k_adamw_apply,
+                                dim3((unsigned)((cols + kCols - 1) / kCols), (unsigned)((rows + kRows - 1) / kRows)),
+                                dim3(kCols), 0, s, W, M, rows, cols, lr, mcorr, eps, lam, inv_rows, colsum);
+    return launch_dependent(k_adamw_mw4<GT>,
+                            dim3((unsigned)((cols / 4 + kCols - 1) / kCols), (unsigned)((rows + kRows2 - 1) / kRows2)),
+                            dim3(kCols), 0, s, g, W, M, rows, cols, b1, lr, mcorr, eps, lam, inv_rows, colsum);
+}
+
 }  // namespace
 
 cudaError_t adamw_rowconst(bool grad_bf16, float *W, const void *g, float *M, float *V,
@@ -207,44 +245,25 @@ cudaError_t adamw_rowconst(bool grad_bf16, float *W, const void *g, float *M, fl
     // three dependent launches: a memset between two kernels would end the overlap
     cudaError_t e = launch_dependent(k_zero, dim3((unsigned)std::min<int64_t>((cols + kCols - 1) / kCols, 152)),
                                      dim3(kCols), 0, s, colsum, cols);
-    if (e != cudaSuccess)
-        return e;
+    count_launch();
     // bias corrections of step t, in double before rounding to fp32
     const float vcorr = (float)(1.0 / (1.0 - pow((double)b2, (double)t)));
     const float mcorr = (float)(1.0 / (1.0 - pow((double)b1, (double)t)));
-    if (cols % 4 == 0) {
-        const dim3 grid((unsigned)((cols / 4 + kCols - 1) / kCols),
-                        (unsigned)((rows + kRowsV - 1) / kRowsV));
-        const float inv_rows = (float)(1.0 / (double)rows);
-        if (grad_bf16) {
-            const __nv_bfloat16 *gp = (const __nv_bfloat16 *)g;
-            e = launch_dependent(k_adamw_v4<__nv_bfloat16>, grid, dim3(kCols), 0, s, gp, V, rows, cols, b2,
-                                 vcorr, colsum);
-            if (e == cudaSuccess)
-                e = launch_dependent(k_adamw_mw4<__nv_bfloat16>, grid, dim3(kCols), 0, s, gp, W, M, rows,
-                                     cols, b1, lr, mcorr, eps, lam, inv_rows, colsum);
-        } else {
-            const float *gp = (const float *)g;
-            e = launch_dependent(k_adamw_v4<float>, grid, dim3(kCols), 0, s, gp, V, rows, cols, b2, vcorr,
-                                 colsum);
-            if (e == cudaSuccess)
-                e = launch_dependent(k_adamw_mw4<float>, grid, dim3(kCols), 0, s, gp, W, M, rows, cols, b1,
-                                     lr, mcorr, eps, lam, inv_rows, colsum);
-        }
-        count_launch(3);
-        return e != cudaSuccess ? e : cudaGetLastError();
+    const float inv_rows = (float)(1.0 / (double)rows);
+    // a grid's y extent holds 65535 blocks: more rows go in several launches per pass
+    const int64_t most = (int64_t)65535 * (cols % 4 == 0 ? kRows2 : kRows);
+    for (int64_t r = 0; r < rows && e == cudaSuccess; r += most) {
+        const int64_t n = std::min(rows - r, most), o = r * cols;
+        e = grad_bf16 ? moments((const __nv_bfloat16 *)g + o, M + o, V + o, n, cols, b1, b2, vcorr, colsum, s)
+                      : moments((const float *)g + o, M + o, V + o, n, cols, b1, b2, vcorr, colsum, s);
     }
-    const dim3 grid((unsigned)((cols + kCols - 1) / kCols), (unsigned)((rows + kRows - 1) / kRows));
-    if (grad_bf16)
-        e = launch_dependent(k_adamw_moments<__nv_bfloat16>, grid, dim3(kCols), 0, s,
-                             (const __nv_bfloat16 *)g, M, V, rows, cols, b1, b2, vcorr, colsum);
-    else
-        e = launch_dependent(k_adamw_moments<float>, grid, dim3(kCols), 0, s, (const float *)g, M, V, rows,
-                             cols, b1, b2, vcorr, colsum);
-    if (e == cudaSuccess)
-        e = launch_dependent(k_adamw_apply, grid, dim3(kCols), 0, s, W, M, rows, cols, lr, mcorr, eps, lam,
-                             (float)(1.0 / (double)rows), colsum);
-    count_launch(3);
+    for (int64_t r = 0; r < rows && e == cudaSuccess; r += most) {
+        const int64_t n = std::min(rows - r, most), o = r * cols;
+        e = grad_bf16 ? apply((const __nv_bfloat16 *)g + o, W + o, M + o, n, cols, b1, lr, mcorr, eps, lam,
+                              inv_rows, colsum, s)
+                      : apply((const float *)g + o, W + o, M + o, n, cols, b1, lr, mcorr, eps, lam, inv_rows,
+                              colsum, s);
+    }
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -89,3 +89,20 @@ def test_adamw_argument_errors(sn):
     with pytest.raises(sn.SNError) as e:
         sn.sn_adamw_rowconst(W, g, M, V, 1, 1e-3, workspace=torch.empty(4, device="cuda"))
     assert e.value.status == sn.SN_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("rows,cols", [(16 * 65535 + 37, 4), (16 * 65535 + 5, 1), (17, 1028), (9, 1024)])
+def test_row_blocks(sn, rows, cols):
+    """More runs of 16 and 8 rows than a grid's y extent holds, and a few rows: one step
+    against the definition in fp64.  M and V carry one rounding; W's rate comes from
+    fp32 column sums, whose error of about 1e-6 moves W by that part of a 1e-3 step."""
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    W, M, grad = (torch.randn(rows, cols, generator=g, device="cuda") for _ in range(3))
+    V = torch.rand(rows, cols, generator=g, device="cuda")
+    M64 = 0.9 * M.double() + 0.1 * grad.double()
+    V64 = 0.95 * V.double() + 0.05 * grad.double() ** 2
+    rate = (V64.mean(0) / (1 - 0.95 ** 2)).sqrt() + 1e-8
+    W64 = W.double() - 1e-3 * (M64 / (1 - 0.9 ** 2)) / rate - 1e-4 * W.double()
+    sn.sn_adamw_rowconst(W, grad, M, V, 2, 1e-3, 0.9, 0.95, 1e-8, 1e-4)
+    for got, want in ((W, W64), (M, M64), (V, V64)):
+        assert float((got.double() - want).norm() / want.norm()) <= 1e-6
