@@ -216,7 +216,11 @@ __global__ void __launch_bounds__(CTHREADS) k_simt_compress(const SimtCompress p
 #pragma unroll
         for (int n = 0; n < TN; ++n)
             acc[m][n] = 0ull;
-    const int tg = lane >> 2, cg = lane & 3;        // token lane, column lane
+    // Token lane, column lane.  A pass of the shared memory serves equal addresses where
+    // neighbouring lanes share them: wide tiles, whose reads of U outweigh those of the
+    // rows, put the lanes of one column side by side (k = 128: 112 us instead of 174).
+    constexpr bool kWide = TN >= 6;
+    const int tg = kWide ? lane & 7 : lane >> 2, cg = kWide ? lane >> 3 : lane & 3;
     const int nch = (p.d + CCH - 1) / CCH, step = p.split * G;
     int c = rank * G + group;
     if (c < nch) {
