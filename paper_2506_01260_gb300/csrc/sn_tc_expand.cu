@@ -13,8 +13,9 @@
 //              buffers (M = 128, N = 128): C U^T over K = k padded to 16;
 //   warps 2-9  two epilogue groups taking alternate blocks: drain the
 //              accumulator 64 columns at a time, round once to bf16 into the
-//              group's swizzled staging tile and write each warp's 32 rows with
-//              coalesced 16-byte stores (the TMA unit is left to the loads);
+//              group's swizzled staging tile; each warp stores its 32 rows with
+//              TMA (T = 16384, d = 4096, k = 41: 26.3 us a call; 28.0 with coalesced
+//              16-byte stores read back from the staging tile);
 //              together the groups repack each item's C rows into the swizzled
 //              K-major A operand (zero-padded).  Stages are released by the MMA
 //              commit.
@@ -239,9 +240,13 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
                 tc_fence_after();
                 // drain the accumulator 64 columns at a time and stage the rounded
                 // values in this group's swizzled staging tile (one [128 x 64]
-                // atom per 64 columns; the warp touches only its own 32 rows)
+                // atom per 64 columns; the warp touches only its own 32 rows, once
+                // its previous stores have read them)
                 const uint32_t slot = out_s + grp * (NB / 64) * kTile;
                 const int c0 = blk * NB;
+                if (lane == 0)
+                    bulk_wait_read0();
+                __syncwarp();
 #pragma unroll
                 for (int h = 0; h < NB / 64; ++h) {
                     float v[64];
@@ -276,24 +281,22 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
                         }
                     }
                 }
+                // the warp's 32 rows leave by TMA, clipped at the tensor's edges
+                fence_async_smem();
                 __syncwarp();
-                // coalesced 16-byte stores: NB / 8 lanes per output row segment
-                constexpr int kCpr = NB / 8, kRpi = 32 / kCpr;
-                const int chunk = lane % kCpr;
-                const bool col_ok = c0 + 8 * chunk + 8 <= p.ncols8;
-                const uint32_t src = slot + (chunk >> 3) * kTile;
+                if (lane == 0 && r0 + 32 * q < p.rows) {
 #pragma unroll
-                for (int i = 0; i < 32 / kRpi; ++i) {
-                    const int rr = 32 * q + kRpi * i + lane / kCpr;
-                    const int64_t t = r0 + rr;
-                    const uint4 o = lds128(src + sw128(rr, chunk & 7));
-                    if (col_ok && t < p.rows)
-                        *(uint4 *)(p.out + t * p.out_ld + c0 + 8 * chunk) = o;
+                    for (int h = 0; h < NB / 64; ++h)
+                        if (c0 + 64 * h < p.ncols8)
+                            tma_store_2d(&p.mapOut, slot + h * kTile + 32 * q * 128, c0 + 64 * h,
+                                         (int)(r0 + 32 * q));
+                    bulk_commit();
                 }
                 __syncwarp();
             }
         }
-
+        if (lane == 0)
+            bulk_wait_all0();
     }
 
     tc_fence_before();
