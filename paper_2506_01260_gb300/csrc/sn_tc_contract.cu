@@ -43,11 +43,11 @@ namespace {
 // (their ids were loaded at chunk 1)
 constexpr int kRowsPrep = 6;
 
-// j-th chunk of an item: every CTA starts at a different chunk so that the
-// CTAs do not all read the same U^T chunk from one L2 slice at once.
-__device__ __forceinline__ int chunk_at(int kc0, int kc1, int j)
+// First chunk of an item's walk (cyclic): every CTA starts at a different chunk so
+// that the CTAs do not all read the same U^T chunk from one L2 slice at once.
+__device__ __forceinline__ int first_chunk(int kc0, int kc1)
 {
-    return kc0 + (int)((j + blockIdx.x) % (kc1 - kc0));
+    return kc0 + (int)(blockIdx.x % (kc1 - kc0));
 }
 
 template <int MODE>
@@ -82,6 +82,10 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
         mbar_init(drain_b, 1);
         *abort_flag = 0;
         mbar_fence_init();
+        tma_prefetch(&p.mapA);
+        tma_prefetch(&p.mapU);
+        if (MODE == CMODE_X && p.has_pe)
+            tma_prefetch(&p.mapPE);
     }
     if (warp == 1)
         tmem_alloc(smem_u32(tmem_slot), tmem_cols);
@@ -95,33 +99,28 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            tma_prefetch(&p.mapA);
-            tma_prefetch(&p.mapU);
-            if (MODE == CMODE_X && p.has_pe)
-                tma_prefetch(&p.mapPE);
-        }
-        uint32_t g = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-            const ItemSpan sp = item_span(p, item);
-            const int tile = sp.tile, kc0 = sp.kc0, kc1 = sp.kc1;
-            const int64_t r0 = MODE == CMODE_W ? (int64_t)tile * BM
-                                               : tile_row0(tile, p.reorder, p.batches, p.seq_len);
-            const bool pe_tile = MODE == CMODE_X && p.has_pe && !p.has_pos &&
-                                 (r0 % p.seq_len) + BM <= p.seq_len;
-            const uint32_t tx = pl.a_bytes + pl.u_bytes + (pe_tile ? kTile : 0);
-            for (int j = 0; j < kc1 - kc0; ++j, ++g) {
-                const int kc = chunk_at(kc0, kc1, j);
-                const int s = g % S;
-                const uint32_t n = g / S;
-                if (!warp_wait(empty_b + 8 * s, (n & 1) ^ 1, abort_flag, p.err)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t st = base + s * pl.stage_bytes;
-                const uint32_t fb = full_b + 8 * s;
-                if (lane == 0) {
+        if (lane == 0) {       // one lane alone: a freed stage is refilled without a warp's votes
+            uint32_t g = 0;
+            Ring ring;
+            bool ok = true;
+            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+                const ItemSpan sp = item_span(p, item);
+                const int tile = sp.tile, kc0 = sp.kc0, kc1 = sp.kc1;
+                const int64_t r0 = MODE == CMODE_W ? (int64_t)tile * BM
+                                                   : tile_row0(tile, p.reorder, p.batches, p.seq_len);
+                const bool pe_tile = MODE == CMODE_X && p.has_pe && !p.has_pos &&
+                                     (r0 % p.seq_len) + BM <= p.seq_len;
+                const int pe_row0 = pe_tile ? (int)(r0 % p.seq_len) : 0;
+                const uint32_t tx = pl.a_bytes + pl.u_bytes + (pe_tile ? kTile : 0);
+                int kc = first_chunk(kc0, kc1);
+                for (int j = 0; j < kc1 - kc0; ++j, ++g, ring.next(S)) {
+                    const uint32_t s = ring.s;
+                    if (!mbar_wait(empty_b + 8 * s, ring.ph ^ 1, abort_flag, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t st = base + s * pl.stage_bytes;
+                    const uint32_t fb = full_b + 8 * s;
                     mbar_arrive_tx(fb, tx);
                     if (MODE == CMODE_W) {   // W[kc*64 .. +64, r0 .. r0+128): d rows x c
                         tma_load_2d(st, &p.mapA, (int)r0, kc * BK, fb);
@@ -131,15 +130,15 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
                     }
                     tma_load_2d(st + pl.a_bytes, &p.mapU, kc * BK, 0, fb);
                     if (pe_tile)
-                        tma_load_2d(st + pl.a_bytes + pl.u_bytes + pl.raw_bytes, &p.mapPE,
-                                    kc * BK, (int)(r0 % p.seq_len), fb);
+                        tma_load_2d(st + pl.a_bytes + pl.u_bytes + pl.raw_bytes, &p.mapPE, kc * BK,
+                                    pe_row0, fb);
+                    if (++kc == kc1)
+                        kc = kc0;
                 }
-                __syncwarp();
             }
-        }
-        if (!ok && lane == 0) {   // let copies already issued land before the CTA exits
-            for (uint32_t i = g > (uint32_t)S ? g - S : 0; i < g; ++i)
-                drain_wait(full_b + 8 * (i % S), (i / S) & 1);
+            if (!ok)               // let copies already issued land before the CTA exits
+                for (uint32_t i = g > (uint32_t)S ? g - S : 0; i < g; ++i)
+                    drain_wait(full_b + 8 * (i % S), (i / S) & 1);
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -147,7 +146,8 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16(BM, p.n_pad, false, MODE == CMODE_W);
             const uint32_t idesc_neg = idesc_bf16(BM, p.n_pad, true);
-            uint32_t g = 0, it = 0;
+            uint32_t it = 0;
+            Ring ring;
             bool ok = true;
             for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
                 const ItemSpan sp = item_span(p, item);
@@ -159,10 +159,9 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
                 }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + b * p.acc_stride;
-                for (int j = 0; j < kc1 - kc0; ++j, ++g) {
-                    const int s = g % S;
-                    const uint32_t n = g / S;
-                    if (!mbar_wait(full_b + 8 * s, n & 1, abort_flag, p.err)) {
+                for (int j = 0; j < kc1 - kc0; ++j, ring.next(S)) {
+                    const uint32_t s = ring.s;
+                    if (!mbar_wait(full_b + 8 * s, ring.ph, abort_flag, p.err)) {
                         ok = false;
                         break;
                     }
@@ -355,7 +354,7 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
     } else if (MODE == CMODE_X) {
         // ------------------------------------------------------------ gather warps
         const int tt = threadIdx.x - 192;    // 0..127
-        uint32_t g = 0;
+        Ring ring;
         bool ok = true;
         // The next item's gather rows (this thread's 8 rows of T_fixed and P)
         // are prepared during the current item, where the gather warps wait for
@@ -416,15 +415,14 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
             const int next_tile =
                 item + (int)gridDim.x < nitems ? item_span(p, item + gridDim.x).tile : -1;
             const int nj = kc1 - kc0;
-            for (int j = 0; j < nj; ++j, ++g) {
+            int kc = first_chunk(kc0, kc1);
+            for (int j = 0; j < nj; ++j, ring.next(S)) {
                 if (j == 1)
                     load_rows(next_tile);
                 else if (j == kRowsPrep)
                     prep_rows();
-                const int kc = chunk_at(kc0, kc1, j);
-                const int s = g % S;
-                const uint32_t n = g / S;
-                if (!warp_wait_relaxed(empty_b + 8 * s, (n & 1) ^ 1, abort_flag, p.err)) {
+                const uint32_t s = ring.s;
+                if (!warp_wait_relaxed(empty_b + 8 * s, ring.ph ^ 1, abort_flag, p.err)) {
                     ok = false;
                     break;
                 }
@@ -433,6 +431,8 @@ __global__ void __launch_bounds__(contract_threads(MODE), 1)
                 if (p.has_pe && !pe_tile)
                     gather_rows_async(tb + pl.raw_bytes, p.pe, prow, (int64_t)kc * BK, p.d, tt);
                 cp_async_arrive(full_b + 8 * s);
+                if (++kc == kc1)
+                    kc = kc0;
             }
             // items too short to reach those chunks
             if (nj <= 1)

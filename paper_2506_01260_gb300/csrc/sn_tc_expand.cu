@@ -30,12 +30,11 @@ namespace sn {
 namespace tc {
 namespace {
 
-// j-th block of an item: every CTA starts at a different block so that the
-// CTAs do not all read the same rows of the B operand from one L2 slice at once.
-__device__ __forceinline__ int block_at(int blk0, int blk1, int j)
+// First block of an item's walk (cyclic): every CTA starts at a different block so
+// that the CTAs do not all read the same rows of the B operand from one L2 slice at once.
+__device__ __forceinline__ int first_block(int blk0, int blk1)
 {
-    const int nb = blk1 - blk0;
-    return blk0 + (int)((j + blockIdx.x) % nb);
+    return blk0 + (int)(blockIdx.x % (blk1 - blk0));
 }
 
 template <int AMODE>
@@ -76,6 +75,10 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
         mbar_init(drain_b, 1);
         *abort_flag = 0;
         mbar_fence_init();
+        tma_prefetch(&p.mapB);
+        tma_prefetch(&p.mapOut);
+        if (AMODE == AMODE_TMA)
+            tma_prefetch(&p.mapA);
     }
     if (warp == 1)
         tmem_alloc(smem_u32(tmem_slot), kTmemCols);
@@ -88,53 +91,44 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
-        if (lane == 0) {
-            tma_prefetch(&p.mapB);
-            if (AMODE == AMODE_TMA)
-                tma_prefetch(&p.mapA);
-        }
-        uint32_t g = 0, it = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
-            const int tile = item / p.chunks, ch = item % p.chunks;
-            const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
-            const int64_t r0 = tile_row0(tile, p.reorder, p.batches, p.seq_len);
-            if (AMODE == AMODE_TMA) {
-                if (!warp_wait(aempty_b, (it & 1) ^ 1, abort_flag, p.err)) {
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) {
+        if (lane == 0) {       // one lane alone: a freed stage is refilled without a warp's votes
+            uint32_t g = 0, it = 0;
+            Ring ring;
+            bool ok = true;
+            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
+                const int tile = item / p.chunks, ch = item % p.chunks;
+                const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
+                const int64_t r0 = tile_row0(tile, p.reorder, p.batches, p.seq_len);
+                if (AMODE == AMODE_TMA) {
+                    if (!mbar_wait(aempty_b, (it & 1) ^ 1, abort_flag, p.err)) {
+                        ok = false;
+                        break;
+                    }
                     mbar_arrive_tx(afull_b, pl.a_bytes);
                     for (int a = 0; a < p.katoms; ++a)
                         tma_load_2d(a_s + a * kTile, &p.mapA, a * 64, (int)r0, afull_b);
                 }
-                __syncwarp();
-            }
-            const uint32_t tx = pl.b_bytes;
-            for (int j = 0; j < blk1 - blk0; ++j, ++g) {
-                const int blk = block_at(blk0, blk1, j);
-                const int s = g % S;
-                const uint32_t n = g / S;
-                if (!warp_wait(empty_b + 8 * s, (n & 1) ^ 1, abort_flag, p.err)) {
-                    ok = false;
-                    break;
-                }
-                const uint32_t st = stage0 + s * pl.stage_bytes;
-                const uint32_t fb = full_b + 8 * s;
-                if (lane == 0) {
-                    mbar_arrive_tx(fb, tx);
+                int blk = first_block(blk0, blk1);
+                for (int j = blk0; j < blk1; ++j, ++g, ring.next(S)) {
+                    if (!mbar_wait(empty_b + 8 * ring.s, ring.ph ^ 1, abort_flag, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t st = stage0 + ring.s * pl.stage_bytes;
+                    const uint32_t fb = full_b + 8 * ring.s;
+                    mbar_arrive_tx(fb, pl.b_bytes);
                     for (int a = 0; a < p.katoms; ++a)
                         tma_load_2d(st + a * (NB * 128), &p.mapB, a * 64, blk * NB, fb);
+                    if (++blk == blk1)
+                        blk = blk0;
                 }
-                __syncwarp();
             }
-        }
-        if (!ok && lane == 0) {
-            for (uint32_t i = g > (uint32_t)S ? g - S : 0; i < g; ++i)
-                drain_wait(full_b + 8 * (i % S), (i / S) & 1);
-            if (AMODE == AMODE_TMA && it > 0)
-                drain_wait(afull_b, (it - 1) & 1);
+            if (!ok) {
+                for (uint32_t i = g > (uint32_t)S ? g - S : 0; i < g; ++i)
+                    drain_wait(full_b + 8 * (i % S), (i / S) & 1);
+                if (AMODE == AMODE_TMA && it > 0)
+                    drain_wait(afull_b, (it - 1) & 1);
+            }
         }
         __syncwarp();
     } else if (warp == 1) {
@@ -142,6 +136,7 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16(BM, NB);
             uint32_t g = 0, it = 0;
+            Ring ring;
             bool ok = true;
             for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
                 const int ch = item % p.chunks;
@@ -151,10 +146,9 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
                     break;
                 }
                 tc_fence_after();
-                for (int j = 0; j < blk1 - blk0; ++j, ++g) {
-                    const int s = g % S;
-                    const uint32_t n = g / S, b = g % kExpandAcc, nb = g / kExpandAcc;
-                    if (!mbar_wait(full_b + 8 * s, n & 1, abort_flag, p.err) ||
+                for (int j = 0; j < blk1 - blk0; ++j, ++g, ring.next(S)) {
+                    const uint32_t s = ring.s, b = g % kExpandAcc, nb = g / kExpandAcc;
+                    if (!mbar_wait(full_b + 8 * s, ring.ph, abort_flag, p.err) ||
                         !mbar_wait(acce_b + 8 * b, (nb & 1) ^ 1, abort_flag, p.err)) {
                         ok = false;
                         break;
@@ -228,10 +222,13 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
                 if (lane == 0)
                     mbar_arrive(afull_b);
             }
+            int next = first_block(blk0, blk1);
             for (int j = 0; j < blk1 - blk0; ++j, ++g) {
+                const int blk = next;
+                if (++next == blk1)
+                    next = blk0;
                 if ((int)(g & 1) != grp)
                     continue;
-                const int blk = block_at(blk0, blk1, j);
                 const uint32_t b = g % kExpandAcc, nb = g / kExpandAcc;
                 if (!warp_wait(accf_b + 8 * b, nb & 1, abort_flag, p.err)) {
                     ok = false;

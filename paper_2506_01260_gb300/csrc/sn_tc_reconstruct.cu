@@ -65,10 +65,10 @@ static_assert(kReconAcc * NB <= (int)kReconACol && kReconACol + 2 * kReconAStrid
 static_assert(kPairAcc * NB <= (int)kPairACol && kPairACol + 2 * 2 * 64 <= kTmemCols,
               "TMEM plan (pairs)");
 
-__device__ __forceinline__ int block_at(int blk0, int blk1, int j)
+// First block of an item's walk (cyclic)
+__device__ __forceinline__ int first_block(int blk0, int blk1)
 {
-    const int nb = blk1 - blk0;
-    return blk0 + (int)((j + blockIdx.x) % nb);
+    return blk0 + (int)(blockIdx.x % (blk1 - blk0));
 }
 
 // acc + P + T_fixed for two adjacent columns, rounded once to bf16
@@ -144,6 +144,10 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
         mbar_init(drain_b, 1);
         *abort_flag = 0;
         mbar_fence_init();
+        tma_prefetch(&p.mapB);
+        tma_prefetch(&p.mapOut);
+        if (p.has_pe)
+            tma_prefetch(&p.mapPE);
     }
     if (warp == 1)
         tmem_alloc(smem_u32(tmem_slot), kTmemCols);
@@ -156,38 +160,38 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
 
     if (warp == 0) {
         // ------------------------------------------------------------ B producer
-        if (lane == 0)
-            tma_prefetch(&p.mapB);
-        uint32_t g = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-            const int ch = item % p.chunks;
-            const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
-            for (int j = 0; j < blk1 - blk0; ++j, ++g) {
-                const int blk = block_at(blk0, blk1, j);
-                const int s = g % SB;
-                if (!warp_wait(bempty_b + 8 * s, ((g / SB) & 1) ^ 1, abort_flag, p.err)) {
-                    ok = false;
-                    break;
-                }
-                if (lane == 0) {
-                    const uint32_t fb = bfull_b + 8 * s, st = b0 + s * pl.b_bytes;
+        if (lane == 0) {       // one lane alone: a freed stage is refilled without a warp's votes
+            uint32_t g = 0;
+            Ring ring;
+            bool ok = true;
+            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+                const int ch = item % p.chunks;
+                const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
+                int blk = first_block(blk0, blk1);
+                for (int j = blk0; j < blk1; ++j, ++g, ring.next(SB)) {
+                    if (!mbar_wait(bempty_b + 8 * ring.s, ring.ph ^ 1, abort_flag, p.err)) {
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t fb = bfull_b + 8 * ring.s, st = b0 + ring.s * pl.b_bytes;
                     mbar_arrive_tx(fb, pl.b_bytes);
                     for (int a = 0; a < p.katoms; ++a)
                         tma_load_2d(st + a * (NB * 128), &p.mapB, a * 64, blk * NB, fb);
+                    if (++blk == blk1)
+                        blk = blk0;
                 }
-                __syncwarp();
             }
+            if (!ok)
+                for (uint32_t i = g > (uint32_t)SB ? g - SB : 0; i < g; ++i)
+                    drain_wait(bfull_b + 8 * (i % SB), (i / SB) & 1);
         }
-        if (!ok && lane == 0)
-            for (uint32_t i = g > (uint32_t)SB ? g - SB : 0; i < g; ++i)
-                drain_wait(bfull_b + 8 * (i % SB), (i / SB) & 1);
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16(BM, NB);
             uint32_t g = 0, it = 0;
+            Ring ring;
             bool ok = true;
             for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
                 const int ch = item % p.chunks;
@@ -199,10 +203,9 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
                 }
                 tc_fence_after();
                 const uint32_t a_tmem = tmem + kReconACol + ab * kReconAStride;
-                for (int j = 0; j < blk1 - blk0; ++j, ++g) {
-                    const int s = g % SB;
-                    const uint32_t b = g % kReconAcc;
-                    if (!mbar_wait(bfull_b + 8 * s, (g / SB) & 1, abort_flag, p.err) ||
+                for (int j = 0; j < blk1 - blk0; ++j, ++g, ring.next(SB)) {
+                    const uint32_t s = ring.s, b = g % kReconAcc;
+                    if (!mbar_wait(bfull_b + 8 * s, ring.ph, abort_flag, p.err) ||
                         !mbar_wait(acce_b + 8 * b, ((g / kReconAcc) & 1) ^ 1, abort_flag, p.err)) {
                         ok = false;
                         break;
@@ -233,6 +236,7 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
         const int grp = (warp - 2) >> 2;     // the group's 64-column half of each block
         const int row = 32 * q + lane;
         uint32_t g = 0;
+        uint32_t es = grp, ph = 0;           // embedding stage of this group's next half, its parity
         bool ok = true;
         // the id (and position) of this thread's row, loaded an item ahead so
         // that an item's start does not wait for them
@@ -286,10 +290,12 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
                 if (bad && ch == 0)
                     atomicOr(p.err, SN_EBIT_BAD_ID);
             }
+            int next = first_block(blk0, blk1);
             for (int j = 0; j < blk1 - blk0 && ok; ++j, ++g) {
-                const int blk = block_at(blk0, blk1, j);
+                const int blk = next;
+                if (++next == blk1)
+                    next = blk0;
                 const uint32_t b = g % kReconAcc;
-                const uint32_t e = 2 * g + grp, es = e % SE, ph = (e / SE) & 1;
                 if (!warp_wait(accf_b + 8 * b, (g / kReconAcc) & 1, abort_flag, p.err)) {
                     ok = false;
                     break;
@@ -350,6 +356,11 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
                 __syncwarp();
                 if (lane == 0)
                     mbar_arrive(eempty_b + 8 * es);
+                es += 2;                     // the other group's half lies between
+                if (es >= (uint32_t)SE) {
+                    es -= SE;
+                    ph ^= 1;
+                }
             }
         }
         if (lane == 0)
@@ -358,9 +369,8 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
         // ------------------------------------------------------------ embedding gathers
         const int tt = threadIdx.x - 320;    // 0..127
         const int arow = 32 * (warp & 3) + lane;   // this thread's TMEM lane (A row)
-        if (tt == 0 && p.has_pe)
-            tma_prefetch(&p.mapPE);
-        uint32_t g = 0, e = 0, it = 0;
+        uint32_t e = 0, it = 0;
+        Ring ring;
         bool ok = true;
         // The next item's gather rows (this thread's 8 rows of T_fixed and P)
         // are prepared during the current item, where the gather warps wait for
@@ -458,9 +468,12 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
             const int64_t nt = (has_next ? tile_row0(next_tile, p.reorder, p.batches, p.seq_len) : 0) + arow;
             uint32_t ha[16];
             int mq = 0, hq = 0;
-            for (int j = 0; j < blk1 - blk0 && ok; ++j, ++g) {
-                const int blk = block_at(blk0, blk1, j);
-                for (int hh = 0; hh < 2; ++hh, ++e, ++hq) {
+            int next = first_block(blk0, blk1);
+            for (int j = 0; j < blk1 - blk0 && ok; ++j) {
+                const int blk = next;
+                if (++next == blk1)
+                    next = blk0;
+                for (int hh = 0; hh < 2; ++hh, ++e, ++hq, ring.next(SE)) {
                     if (hq == 1)
                         load_rows(next_tile);
                     else if (hq == kRowsPrep)
@@ -479,8 +492,8 @@ __global__ void __launch_bounds__(kReconThreads, 1) k_reconstruct(const __grid_c
                         load_c_words(p, nt, 16 * mq, ha);
                         ++mq;
                     }
-                    const uint32_t es = e % SE;
-                    if (!warp_wait_relaxed(eempty_b + 8 * es, ((e / SE) & 1) ^ 1, abort_flag, p.err)) {
+                    const uint32_t es = ring.s;
+                    if (!warp_wait_relaxed(eempty_b + 8 * es, ring.ph ^ 1, abort_flag, p.err)) {
                         ok = false;
                         break;
                     }
@@ -607,6 +620,9 @@ __global__ void __launch_bounds__(kReconThreads, 1)
         mbar_init(drain_b, 1);
         *abort_flag = 0;
         mbar_fence_init();
+        tma_prefetch(&p.mapA);
+        tma_prefetch(&p.mapOut);
+        tma_prefetch(&p.mapPE);
     }
     if (warp == 1)
         tmem_alloc(smem_u32(tmem_slot), kTmemCols);
@@ -619,40 +635,40 @@ __global__ void __launch_bounds__(kReconThreads, 1)
 
     if (warp == 0) {
         // ------------------------------------------------------------ B producer
-        if (lane == 0)
-            tma_prefetch(&p.mapA);
-        uint32_t g = 0;
-        bool ok = true;
-        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
-            const int ch = item % p.chunks;
-            const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
-            for (int j = 0; j < blk1 - blk0 && ok; ++j) {
-                const int blk = block_at(blk0, blk1, j);
-                for (int hh = 0; hh < 2; ++hh, ++g) {
-                    const int s = g % SB;
-                    if (!warp_wait(bempty_b + 8 * s, ((g / SB) & 1) ^ 1, abort_flag, p.err)) {
-                        ok = false;
-                        break;
-                    }
-                    if (lane == 0) {
-                        const uint32_t fb = bfull_b + 8 * s, st = b0 + s * pl.b_bytes;
+        if (lane == 0) {       // one lane alone, as in the single-tile form
+            uint32_t g = 0;
+            Ring ring;
+            bool ok = true;
+            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+                const int ch = item % p.chunks;
+                const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
+                int blk = first_block(blk0, blk1);
+                for (int j = blk0; j < blk1 && ok; ++j) {
+                    for (int hh = 0; hh < 2; ++hh, ++g, ring.next(SB)) {
+                        if (!mbar_wait(bempty_b + 8 * ring.s, ring.ph ^ 1, abort_flag, p.err)) {
+                            ok = false;
+                            break;
+                        }
+                        const uint32_t fb = bfull_b + 8 * ring.s, st = b0 + ring.s * pl.b_bytes;
                         mbar_arrive_tx(fb, pl.b_bytes);
                         for (int a = 0; a < p.katoms; ++a)
                             tma_load_2d(st + a * (64 * 128), &p.mapA, a * 64, blk * NB + 64 * hh, fb);
                     }
-                    __syncwarp();
+                    if (++blk == blk1)
+                        blk = blk0;
                 }
             }
+            if (!ok)
+                for (uint32_t i = g > (uint32_t)SB ? g - SB : 0; i < g; ++i)
+                    drain_wait(bfull_b + 8 * (i % SB), (i / SB) & 1);
         }
-        if (!ok && lane == 0)
-            for (uint32_t i = g > (uint32_t)SB ? g - SB : 0; i < g; ++i)
-                drain_wait(bfull_b + 8 * (i % SB), (i / SB) & 1);
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t idesc = idesc_bf16(BM, 64);
             uint32_t g = 0, it = 0;
+            Ring ring;
             bool ok = true;
             for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
                 const int ch = item % p.chunks;
@@ -665,10 +681,9 @@ __global__ void __launch_bounds__(kReconThreads, 1)
                 tc_fence_after();
                 const uint32_t a_tmem = tmem + kPairACol + ab * 2 * aw;
                 for (int j = 0; j < blk1 - blk0 && ok; ++j) {
-                    for (int hh = 0; hh < 2; ++hh, ++g) {
-                        const int s = g % SB;
-                        const uint32_t b = g % kPairAcc;
-                        if (!mbar_wait(bfull_b + 8 * s, (g / SB) & 1, abort_flag, p.err) ||
+                    for (int hh = 0; hh < 2; ++hh, ++g, ring.next(SB)) {
+                        const uint32_t s = ring.s, b = g % kPairAcc;
+                        if (!mbar_wait(bfull_b + 8 * s, ring.ph, abort_flag, p.err) ||
                             !mbar_wait(acce_b + 8 * b, ((g / kPairAcc) & 1) ^ 1, abort_flag, p.err)) {
                             ok = false;
                             break;
@@ -703,6 +718,7 @@ __global__ void __launch_bounds__(kReconThreads, 1)
         const int grp = (warp - 2) >> 2;     // the group's tile of the pair
         const int row = 32 * q + lane;
         uint32_t g = 0;
+        Ring ring;
         bool ok = true;
         // the id of this thread's row, loaded an item ahead
         int nid = 0;
@@ -750,11 +766,14 @@ __global__ void __launch_bounds__(kReconThreads, 1)
                 if (bad && ch == 0)
                     atomicOr(p.err, SN_EBIT_BAD_ID);
             }
+            int next = first_block(blk0, blk1);
             for (int j = 0; j < blk1 - blk0 && ok; ++j) {
-                const int blk = block_at(blk0, blk1, j);
-                for (int hh = 0; hh < 2; ++hh, ++g) {
+                const int blk = next;
+                if (++next == blk1)
+                    next = blk0;
+                for (int hh = 0; hh < 2; ++hh, ++g, ring.next(SE)) {
                     const uint32_t b = g % kPairAcc;
-                    const uint32_t es = g % SE, ph = (g / SE) & 1;
+                    const uint32_t es = ring.s, ph = ring.ph;
                     if (!warp_wait(accf_b + 8 * b, (g / kPairAcc) & 1, abort_flag, p.err)) {
                         ok = false;
                         break;
@@ -816,9 +835,8 @@ __global__ void __launch_bounds__(kReconThreads, 1)
         // ------------------------------------------------------------ gathers and A
         const int tt = threadIdx.x - 320;    // 0..127
         const int arow = 32 * (warp & 3) + lane;   // this thread's TMEM lane (A row)
-        if (tt == 0)
-            tma_prefetch(&p.mapPE);
         uint32_t e = 0, it = 0;
+        Ring ring;
         bool ok = true;
         // T_fixed rows of this thread's 8 rows of each tile for the next item,
         // loaded one half block into the current item and checked a few later
@@ -890,9 +908,12 @@ __global__ void __launch_bounds__(kReconThreads, 1)
             const int64_t nr0 = has_next ? pair_row0(next_pp, p.batches, p.seq_len) : 0;
             uint32_t ha[16];
             int mq = 0, hq = 0;
+            int next = first_block(blk0, blk1);
             for (int j = 0; j < blk1 - blk0 && ok; ++j) {
-                const int blk = block_at(blk0, blk1, j);
-                for (int hh = 0; hh < 2; ++hh, ++e, ++hq) {
+                const int blk = next;
+                if (++next == blk1)
+                    next = blk0;
+                for (int hh = 0; hh < 2; ++hh, ++e, ++hq, ring.next(SE)) {
                     if (hq == 1)
                         load_rows(next_pp);
                     else if (hq == kRowsPrep)
@@ -912,8 +933,8 @@ __global__ void __launch_bounds__(kReconThreads, 1)
                         load_c_words(p, nr0 + (int64_t)(mq / nch) * p.seq_len + arow, 16 * (mq % nch), ha);
                         ++mq;
                     }
-                    const uint32_t es = e % SE;
-                    if (!warp_wait_relaxed(eempty_b + 8 * es, ((e / SE) & 1) ^ 1, abort_flag, p.err)) {
+                    const uint32_t es = ring.s;
+                    if (!warp_wait_relaxed(eempty_b + 8 * es, ring.ph ^ 1, abort_flag, p.err)) {
                         ok = false;
                         break;
                     }
