@@ -16,9 +16,15 @@
 //              group's swizzled staging tile; each warp stores its 32 rows with
 //              TMA (T = 16384, d = 4096, k = 41: 26.3 us a call; 28.0 with coalesced
 //              16-byte stores read back from the staging tile);
-//              together the groups repack each item's C rows into the swizzled
+//              together the groups repack the first item's C rows into the swizzled
 //              K-major A operand (zero-padded).  Stages are released by the MMA
-//              commit.
+//              commit;
+//   warps 10-13  (only where a CTA runs several items) repack every later item's C
+//              rows into the other of two A buffers while the MMAs still read the
+//              first: done by the epilogue groups between two items, each change of
+//              item left the stores idle for 3.7 us (T = 65536, d = 8192, k = 81, seven
+//              items a CTA: 204.7 us a call, now 184; the same bytes stored without any
+//              computation took 162 to 174).
 // Each CTA walks an item's blocks starting at its own offset, so the CTAs'
 // B-operand reads are spread over the L2 instead of converging on one slice.
 // Every wait is bounded (SN_EBIT_TIMEOUT); an aborting CTA drains its copies
@@ -37,8 +43,38 @@ __device__ __forceinline__ int first_block(int blk0, int blk1)
     return blk0 + (int)(blockIdx.x % (blk1 - blk0));
 }
 
+// A operand: rows r0 .. r0+127 of C, zero-padded to katoms * 64 columns, into the
+// swizzled K-major tile at `dst`.  Thread tt takes, of row tt, atom `half` (two atoms)
+// or chunks 4 half .. 4 half + 3 (one atom), issuing all loads before the first use.
+__device__ __forceinline__ void repack_half(const ExpandParams &p, int64_t r0, int tt, int half,
+                                            uint32_t dst)
+{
+    const int64_t t = r0 + tt;
+    const int a = p.katoms == 2 ? half : 0;
+    const int cbeg = p.katoms == 2 ? 0 : 4 * half;
+    const int jbeg = a * 64 + cbeg * 8;
+    const unsigned short *crow = (const unsigned short *)p.C + t * p.k;
+    uint32_t h[32];
+#pragma unroll
+    for (int e = 0; e < 32; ++e) {
+        const int j0 = jbeg + 2 * e;
+        // one atom covers 64 columns: with two atoms each thread takes
+        // 32 words, with one atom 16 words
+        const bool want = (p.katoms == 2 || e < 16) && t < p.rows;
+        const uint32_t lo = (want && j0 < p.k) ? __ldg(crow + j0) : 0u;
+        const uint32_t hi = (want && j0 + 1 < p.k) ? __ldg(crow + j0 + 1) : 0u;
+        h[e] = lo | (hi << 16);
+    }
+    const int nchunks = p.katoms == 2 ? 8 : 4;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        if (c < nchunks)
+            sts128(dst + a * kTile + sw128(tt, cbeg + c),
+                   make_uint4(h[4 * c], h[4 * c + 1], h[4 * c + 2], h[4 * c + 3]));
+}
+
 template <int AMODE>
-__global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_constant__ ExpandParams p)
+__global__ void __launch_bounds__(expand_threads(AMODE), 1) k_expand(const __grid_constant__ ExpandParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     uint32_t base = smem_u32(smem_raw);
@@ -48,14 +84,14 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
 
     const int S = p.stages;
     const ExpandPlan pl = expand_plan(p.katoms, S);
-    const uint32_t a_s = base, out_s = base + pl.a_bytes;
+    const uint32_t a_s = base, out_s = base + 2 * pl.a_bytes;
     const uint32_t stage0 = out_s + pl.out_bytes;
     const uint32_t bar = base + pl.bar_off;
     const uint32_t full_b = bar, empty_b = bar + 8 * S;
     const uint32_t accf_b = bar + 16 * S, acce_b = accf_b + 8 * kExpandAcc;
-    const uint32_t afull_b = acce_b + 8 * kExpandAcc, aempty_b = afull_b + 8;
-    const uint32_t drain_b = aempty_b + 8;
-    uint32_t *tmem_slot = (uint32_t *)(smem + pl.bar_off + 8 * (2 * S + 2 * kExpandAcc + 3));
+    const uint32_t afull_b = acce_b + 8 * kExpandAcc, aempty_b = afull_b + 16;
+    const uint32_t drain_b = aempty_b + 16;
+    uint32_t *tmem_slot = (uint32_t *)(smem + pl.bar_off + 8 * (2 * S + 2 * kExpandAcc + 5));
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int NB = BN_WIDE;
@@ -70,8 +106,10 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
             mbar_init(accf_b + 8 * b, 1);
             mbar_init(acce_b + 8 * b, 4);
         }
-        mbar_init(afull_b, AMODE == AMODE_REPACK ? 8 : 1);
-        mbar_init(aempty_b, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(afull_b + 8 * b, AMODE == AMODE_REPACK ? 8 : 1);
+            mbar_init(aempty_b + 8 * b, 1);
+        }
         mbar_init(drain_b, 1);
         *abort_flag = 0;
         mbar_fence_init();
@@ -100,13 +138,14 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
                 const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
                 const int64_t r0 = tile_row0(tile, p.reorder, p.batches, p.seq_len);
                 if (AMODE == AMODE_TMA) {
-                    if (!mbar_wait(aempty_b, (it & 1) ^ 1, abort_flag, p.err)) {
+                    const uint32_t ab = it & 1, fb = afull_b + 8 * ab;
+                    if (!mbar_wait(aempty_b + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag, p.err)) {
                         ok = false;
                         break;
                     }
-                    mbar_arrive_tx(afull_b, pl.a_bytes);
+                    mbar_arrive_tx(fb, pl.a_bytes);
                     for (int a = 0; a < p.katoms; ++a)
-                        tma_load_2d(a_s + a * kTile, &p.mapA, a * 64, (int)r0, afull_b);
+                        tma_load_2d(a_s + ab * pl.a_bytes + a * kTile, &p.mapA, a * 64, (int)r0, fb);
                 }
                 int blk = first_block(blk0, blk1);
                 for (int j = blk0; j < blk1; ++j, ++g, ring.next(S)) {
@@ -126,8 +165,9 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
             if (!ok) {
                 for (uint32_t i = g > (uint32_t)S ? g - S : 0; i < g; ++i)
                     drain_wait(full_b + 8 * (i % S), (i / S) & 1);
-                if (AMODE == AMODE_TMA && it > 0)
-                    drain_wait(afull_b, (it - 1) & 1);
+                if (AMODE == AMODE_TMA)
+                    for (uint32_t i = it > 2 ? it - 2 : 0; i < it; ++i)
+                        drain_wait(afull_b + 8 * (i & 1), (i >> 1) & 1);
             }
         }
         __syncwarp();
@@ -141,7 +181,8 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
             for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
                 const int ch = item % p.chunks;
                 const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
-                if (!mbar_wait(afull_b, it & 1, abort_flag, p.err)) {
+                const uint32_t ab = it & 1, a_it = a_s + ab * pl.a_bytes;
+                if (!mbar_wait(afull_b + 8 * ab, (it >> 1) & 1, abort_flag, p.err)) {
                     ok = false;
                     break;
                 }
@@ -158,14 +199,14 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
                     const uint32_t d_tmem = tmem + b * NB;
                     for (int kk = 0; kk < p.kmma; ++kk) {
                         const uint32_t a = kk >> 2, off = (kk & 3) * 32;
-                        mma_bf16(d_tmem, sdesc_sw128(a_s + a * kTile + off),
+                        mma_bf16(d_tmem, sdesc_sw128(a_it + a * kTile + off),
                                  sdesc_sw128(st + a * (NB * 128) + off), idesc, kk > 0 ? 1u : 0u);
                     }
                     mma_commit(empty_b + 8 * s);     // stage free once these MMAs finish
                     mma_commit(accf_b + 8 * b);
                 }
                 if (ok)
-                    mma_commit(aempty_b);
+                    mma_commit(aempty_b + 8 * ab);
             }
             if (!ok) {
                 mma_commit(drain_b);
@@ -179,49 +220,20 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
         const int grp = (warp - 2) >> 2;     // blocks g with g % 2 == grp
         const int tt = 32 * ((warp - 2) & 3) + lane;   // 0..127 within the group
         const int row = 32 * q + lane;
-        uint32_t g = 0, it = 0;
+        uint32_t g = 0;
         bool ok = true;
-        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x, ++it) {
+        if (AMODE == AMODE_REPACK && (int)blockIdx.x < nitems) {   // the first item's A rows
+            repack_half(p, tile_row0(blockIdx.x / p.chunks, p.reorder, p.batches, p.seq_len), tt, grp,
+                        a_s);
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(afull_b);
+        }
+        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
             const int tile = item / p.chunks, ch = item % p.chunks;
             const int blk0 = ch * p.bpi, blk1 = min(blk0 + p.bpi, p.nblk);
             const int64_t r0 = tile_row0(tile, p.reorder, p.batches, p.seq_len);
-            if (AMODE == AMODE_REPACK) {
-                // A operand: rows r0 .. r0+127 of C, zero-padded to katoms * 64
-                // columns.  Both groups share it: thread (r, half) covers atom
-                // `half` (two atoms) or chunks 4 half .. 4 half + 3 (one atom) of
-                // row r, issuing all of its loads before the first use.
-                if (!warp_wait(aempty_b, (it & 1) ^ 1, abort_flag, p.err)) {
-                    ok = false;
-                    break;
-                }
-                const int r = tt, half = grp;
-                const int64_t t = r0 + r;
-                const int a = p.katoms == 2 ? half : 0;
-                const int cbeg = p.katoms == 2 ? 0 : 4 * half;
-                const int jbeg = a * 64 + cbeg * 8;
-                const unsigned short *crow = (const unsigned short *)p.C + t * p.k;
-                uint32_t h[32];
-#pragma unroll
-                for (int e = 0; e < 32; ++e) {
-                    const int j0 = jbeg + 2 * e;
-                    // one atom covers 64 columns: with two atoms each thread takes
-                    // 32 words, with one atom 16 words
-                    const bool want = (p.katoms == 2 || e < 16) && t < p.rows;
-                    const uint32_t lo = (want && j0 < p.k) ? __ldg(crow + j0) : 0u;
-                    const uint32_t hi = (want && j0 + 1 < p.k) ? __ldg(crow + j0 + 1) : 0u;
-                    h[e] = lo | (hi << 16);
-                }
-                const int nchunks = p.katoms == 2 ? 8 : 4;
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c < nchunks)
-                        sts128(a_s + a * kTile + sw128(r, cbeg + c),
-                               make_uint4(h[4 * c], h[4 * c + 1], h[4 * c + 2], h[4 * c + 3]));
-                fence_async_smem();
-                __syncwarp();
-                if (lane == 0)
-                    mbar_arrive(afull_b);
-            }
             int next = first_block(blk0, blk1);
             for (int j = 0; j < blk1 - blk0; ++j, ++g) {
                 const int blk = next;
@@ -294,6 +306,24 @@ __global__ void __launch_bounds__(kExpandThreads, 1) k_expand(const __grid_const
         }
         if (lane == 0)
             bulk_wait_all0();
+    } else {
+        // ------------------------------------------------------------ A warps
+        // the A rows of every later item, an item ahead of the MMAs
+        const int tt = threadIdx.x - 320;
+        uint32_t it = 1;
+        for (int item = blockIdx.x + gridDim.x; item < nitems; item += gridDim.x, ++it) {
+            const uint32_t ab = it & 1;
+            if (!warp_wait_relaxed(aempty_b + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag, p.err))
+                break;
+            const int64_t r0 = tile_row0(item / p.chunks, p.reorder, p.batches, p.seq_len);
+#pragma unroll 1
+            for (int half = 0; half < 2; ++half)
+                repack_half(p, r0, tt, half, a_s + ab * pl.a_bytes);
+            fence_async_smem();
+            __syncwarp();
+            if (lane < 2)
+                mbar_arrive(afull_b + 8 * ab);
+        }
     }
 
     tc_fence_before();
@@ -310,10 +340,12 @@ cudaError_t launch_expand(int amode, const ExpandParams &p, int grid, cudaStream
 {
     const ExpandPlan pl = expand_plan(p.katoms, p.stages);
     void (*const kernel)(ExpandParams) = amode == AMODE_REPACK ? k_expand<AMODE_REPACK> : k_expand<AMODE_TMA>;
+    // the A warps only serve CTAs that run several items
+    const int threads = p.ntiles * p.chunks > grid ? expand_threads(amode) : kExpandThreads;
     cudaError_t e =
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.total);
     if (e == cudaSuccess)
-        e = launch_dependent(kernel, dim3(grid), dim3(kExpandThreads), pl.total, s, p);
+        e = launch_dependent(kernel, dim3(grid), dim3(threads), pl.total, s, p);
     if (e != cudaSuccess)
         return e;
     count_launch();

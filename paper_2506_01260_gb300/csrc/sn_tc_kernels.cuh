@@ -143,15 +143,20 @@ struct ExpandParams {
 };
 
 // warp 0 producer, warp 1 MMA, warps 2-5 and 6-9 two epilogue groups
-// (alternate blocks)
+// (alternate blocks); then warps 10-13 for the A rows of later items where they
+// do not come by TMA
 constexpr int kExpandThreads = 320;
+__host__ __device__ constexpr int expand_threads(int amode)
+{
+    return amode == AMODE_REPACK ? kExpandThreads + 128 : kExpandThreads;
+}
 constexpr int kExpandAcc = 4;     // TMEM accumulator buffers of 128 columns
 
 struct ExpandPlan {
     uint32_t a_bytes, out_bytes, b_bytes, stage_bytes, bar_off, total;
 };
 
-// Shared memory of the plain expansion: A operand | two output staging tiles |
+// Shared memory of the plain expansion: two A operands | two output staging tiles |
 // stages of B rows | barriers.  A stage is released by the MMA commit; outputs
 // have their own staging, so the stores never hold back the loads.
 __host__ __device__ inline ExpandPlan expand_plan(int katoms, int stages)
@@ -161,8 +166,8 @@ __host__ __device__ inline ExpandPlan expand_plan(int katoms, int stages)
     p.out_bytes = 2 * BM * BN_WIDE * 2;           // one staging tile per epilogue group
     p.b_bytes = (uint32_t)katoms * BN_WIDE * 128;
     p.stage_bytes = p.b_bytes;
-    p.bar_off = p.a_bytes + p.out_bytes + (uint32_t)stages * p.stage_bytes;
-    p.total = p.bar_off + 8 * (2 * stages + 2 * kExpandAcc + 3) + 16 + 1024;
+    p.bar_off = 2 * p.a_bytes + p.out_bytes + (uint32_t)stages * p.stage_bytes;
+    p.total = p.bar_off + 8 * (2 * stages + 2 * kExpandAcc + 5) + 16 + 1024;
     return p;
 }
 
