@@ -215,9 +215,14 @@ __global__ void __launch_bounds__(kThreads) k_topk(const uint16_t *__restrict__ 
         }
         int bound = -1;
         if (M > 0 && q <= 32) {
+            // (the lanes' values agree above their first differing bit, and a bound
+            // up to 3 keys low only admits a few more candidates)
             const int vl = top[M > 0 ? M - 1 : 0];
-            int b = 0;
-            for (int bit = 14; bit >= 0; --bit)
+            const int hi = max(__reduce_max_sync(0xffffffffu, vl), 0);
+            const int lo = max(__reduce_min_sync(0xffffffffu, vl), 0);
+            int bit = 31 - __clz(lo ^ hi);
+            int b = hi & ~((1 << (bit + 1)) - 1);
+            for (; bit >= 2; --bit)
                 if (warp_count(vl >= (b | (1 << bit))) >= q)
                     b |= 1 << bit;
             bound = warp_count(vl >= b) >= q ? b : -1;
@@ -268,19 +273,28 @@ __global__ void __launch_bounds__(kThreads) k_topk(const uint16_t *__restrict__ 
         // every entry at or above the bound is a candidate, so for any trial
         // the candidate count decides "at least kk entries reach it" as the
         // whole row would
-        int thr = 0;
-        for (int bit = 14; bit >= 0; --bit) {
-            const int trial = thr | (1 << bit);
-            int cnt = 0;
-            for (int j = lane; j < nc; j += 32)
-                cnt += (int)(cand[j] & 0x7FFFu) >= trial;
-            if (__reduce_add_sync(0xffffffffu, cnt) >= kk)
-                thr = trial;
-        }
-        int above = 0;
-        for (int j = lane; j < nc; j += 32)
-            above += (int)(cand[j] & 0x7FFFu) > thr;
-        const int need = kk - __reduce_add_sync(0xffffffffu, above);
+        // (the first 64 candidates' keys stay in registers; thr lies between the
+        // bound and the row's largest key, so their common bits are not searched:
+        // with the same shortcut for the bound above, T = 16384, d = 4096, kk = 20
+        // took 48 -> 40 us; two full searches were a third of a row's time)
+        const int key0 = lane < nc ? (int)(cand[lane] & 0x7FFFu) : -1;
+        const int key1 = lane + 32 < nc ? (int)(cand[lane + 32] & 0x7FFFu) : -1;
+        auto reach = [&](int trial) {
+            int cnt = warp_count(key0 >= trial) + warp_count(key1 >= trial);
+            for (int j = 64 + lane; j < nc + lane; j += 32)               // warp-uniform
+                cnt += warp_count(j < nc && (int)(cand[j] & 0x7FFFu) >= trial);
+            return cnt;
+        };
+        int rmax = max(key0, key1);
+        for (int j = 64 + lane; j < nc; j += 32)
+            rmax = max(rmax, (int)(cand[j] & 0x7FFFu));
+        rmax = __reduce_max_sync(0xffffffffu, rmax);
+        int bit = 31 - __clz(rmax ^ max(bound, 0));
+        int thr = rmax & ~((1 << (bit + 1)) - 1);
+        for (; bit >= 0; --bit)
+            if (reach(thr | (1 << bit)) >= kk)
+                thr |= 1 << bit;
+        const int need = kk - reach(thr + 1);
         int eq_before = 0, kept_before = 0;
         for (int r0 = 0; r0 < nc; r0 += 32) {                 // warp-uniform
             const int j = r0 + lane;
