@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kThreads) k_topk(const uint16_t *__restrict__ 
         // (the first 64 candidates' keys stay in registers; thr lies between the
         // bound and the row's largest key, so their common bits are not searched:
         // with the same shortcut for the bound above, T = 16384, d = 4096, kk = 20
-        // took 48 -> 40 us; two full searches were a third of a row's time)
+        // took 48 -> 40 us)
         const int key0 = lane < nc ? (int)(cand[lane] & 0x7FFFu) : -1;
         const int key1 = lane + 32 < nc ? (int)(cand[lane + 32] & 0x7FFFu) : -1;
         auto reach = [&](int trial) {
