@@ -165,8 +165,8 @@ __device__ __forceinline__ bool warp_wait_relaxed(uint32_t bar, uint32_t parity,
 // dividing a running count by the number of stages at every step, and in a producer
 // asking a whole warp to agree on each wait, held the chunk rate of the kernels below
 // the memory's. One step of boundary calls, T x d x k, with divisions and warp-wide
-// producers -> now: 65536 x 8192 x 81 1075 -> 1010 us, 16384 x 4096 x 41 183 -> 175,
-// 4173 x 2056 x 33 packed 54.1 -> 50.5; projection of 4096 x (14336 + 4096), k = 40,
+// producers -> now: 65536 x 8192 x 82 1075 -> 1010 us, 16384 x 4096 x 41 183 -> 175,
+// 4173 x 2056 x 33 packed 54.1 -> 50.5; projection of 4096 x (14336 + 4096), k = 41,
 // 80.6 -> 73.9; compression with a projected operand, 16384 x 4096 x 41, 31.5 -> 26.1.
 struct Ring {
     uint32_t s = 0, ph = 0;

@@ -22,7 +22,7 @@
 //   warps 10-13  (only where a CTA runs several items) repack every later item's C
 //              rows into the other of two A buffers while the MMAs still read the
 //              first: done by the epilogue groups between two items, each change of
-//              item left the stores idle for 3.7 us (T = 65536, d = 8192, k = 81, seven
+//              item left the stores idle for 3.7 us (T = 65536, d = 8192, k = 82, seven
 //              items a CTA: 204.7 us a call, now 184; the same bytes stored without any
 //              computation took 162 to 174).
 // Each CTA walks an item's blocks starting at its own offset, so the CTAs'
