@@ -313,7 +313,8 @@ __global__ void __launch_bounds__(expand_threads(AMODE), 1) k_expand(const __gri
         uint32_t it = 1;
         for (int item = blockIdx.x + gridDim.x; item < nitems; item += gridDim.x, ++it) {
             const uint32_t ab = it & 1;
-            if (!warp_wait_relaxed(aempty_b + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag, p.err))
+            // every lane observes the MMAs' release before it writes over what they read
+            if (!warp_wait(aempty_b + 8 * ab, ((it >> 1) & 1) ^ 1, abort_flag, p.err))
                 break;
             const int64_t r0 = tile_row0(item / p.chunks, p.reorder, p.batches, p.seq_len);
 #pragma unroll 1
