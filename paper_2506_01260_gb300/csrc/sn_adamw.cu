@@ -20,8 +20,38 @@
 namespace sn {
 namespace {
 
-constexpr int kCols = 256;   // columns per block (one per thread)
-constexpr int kRows = 16;    // rows per block
+constexpr int kThreads = 256;
+constexpr int kCols = 256;   // columns per block of the second pass (one per thread)
+constexpr int kRows = 16;    // rows per thread
+
+// The first pass's blocks: kLanes threads along the columns, kGroups groups of them along
+// the rows, each thread kRows rows.  A block's column sums meet in shared memory, so
+// a column takes one atomic for kGroups * kRows = 64 rows: the rounding of the atomic
+// chain is what the sums' error consists of.  One atomic for 16 rows (blocks of 256 x 16)
+// took as long, but its error against 64 bits was 1.6 to 1.8 times as large ([8192, 1024], W = 0:
+// 1.88e-7 of W instead of 1.15e-7).
+constexpr int kLanes = 64, kGroups = kThreads / kLanes;
+
+__device__ __forceinline__ float add(float a, float b) { return a + b; }
+__device__ __forceinline__ float4 add(float4 a, float4 b)
+{
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+// The sum of `s` over the block's row groups, for the threads of the first one
+template <typename T>
+__device__ __forceinline__ T sum_groups(T s)
+{
+    __shared__ T red[kThreads];
+    red[threadIdx.x] = s;
+#pragma unroll
+    for (int o = kThreads / 2; o >= kLanes; o /= 2) {
+        __syncthreads();
+        if ((int)threadIdx.x < o)
+            red[threadIdx.x] = s = add(s, red[threadIdx.x + o]);
+    }
+    return s;
+}
 
 __global__ void __launch_bounds__(kCols) k_zero(float *__restrict__ p, int64_t n)
 {
@@ -44,18 +74,16 @@ __device__ __forceinline__ float load_grad<__nv_bfloat16>(const __nv_bfloat16 *g
 }
 
 template <typename GT>
-__global__ void __launch_bounds__(kCols) k_adamw_moments(const GT *__restrict__ g,
-                                                          float *__restrict__ M,
-                                                          float *__restrict__ V, int64_t rows,
-                                                          int64_t cols, float b1, float b2,
-                                                          float vcorr, float *__restrict__ colsum)
+__global__ void __launch_bounds__(kThreads) k_adamw_moments(const GT *__restrict__ g,
+                                                             float *__restrict__ M,
+                                                             float *__restrict__ V, int64_t rows,
+                                                             int64_t cols, float b1, float b2,
+                                                             float vcorr, float *__restrict__ colsum)
 {
     griddep_wait();
-    const int64_t c = (int64_t)blockIdx.x * kCols + threadIdx.x;
-    const int64_t r0 = (int64_t)blockIdx.y * kRows;
-    if (c >= cols)
-        return;
-    const int64_t r1 = r0 + kRows < rows ? r0 + kRows : rows;
+    const int64_t c = (int64_t)blockIdx.x * kLanes + threadIdx.x % kLanes;
+    const int64_t r0 = ((int64_t)blockIdx.y * kGroups + threadIdx.x / kLanes) * kRows;
+    const int64_t r1 = c < cols ? (r0 + kRows < rows ? r0 + kRows : rows) : 0;
     float s = 0.f;
     for (int64_t r = r0; r < r1; ++r) {
         const int64_t e = r * cols + c;
@@ -66,7 +94,9 @@ __global__ void __launch_bounds__(kCols) k_adamw_moments(const GT *__restrict__ 
         V[e] = v;
         s += v * vcorr;
     }
-    atomicAdd(colsum + c, s);
+    s = sum_groups(s);
+    if (threadIdx.x < kLanes && c < cols)
+        atomicAdd(colsum + c, s);
 }
 
 __global__ void __launch_bounds__(kCols) k_adamw_apply(float *__restrict__ W,
@@ -107,28 +137,26 @@ __device__ __forceinline__ float4 load_grad4<__nv_bfloat16>(const __nv_bfloat16 
                        __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
 }
 
-// Rows per block and rows in flight of the two passes.  Blocks run column-major over a
-// few rows, so the GPU as a whole sweeps the arrays in order of address; the first
-// pass needs enough rows to pay for its atomics.  [4096, 14336], bf16 gradient: blocks of
+// Rows per thread and rows in flight of the two passes.  Blocks run column-major over a
+// few rows, so the GPU as a whole sweeps the arrays in order of address.  [4096, 14336],
+// bf16 gradient: threads of
 // 64 / 32 / 16 + 8 rows take 259 / 251 / 240 us (6.9 TB/s on 28 bytes an element), 8 + 8
 // rows 241, 4 + 4 rows 267; [1024, 1024]: 30 us with 64 rows (64 blocks), 13 with 16 + 8.
 // Evict-first hints on V, M and W or a reversed second pass, to find g in L2, made it
 // slower (262-271 us), and so did a single kernel of clusters that own 128 columns
 // (339), or a loop over several runs of rows in a block (263).
-constexpr int kRows1 = 16, kRows2 = 8;
+constexpr int kRows2 = 8;   // second pass (the first: kRows)
 constexpr int kUnroll1 = 4, kUnroll2 = 8;
 
 template <typename GT>
-__global__ void __launch_bounds__(kCols) k_adamw_v4(const GT *__restrict__ g, float *__restrict__ V,
-                                                     int64_t rows, int64_t cols, float b2, float vcorr,
-                                                     float *__restrict__ colsum)
+__global__ void __launch_bounds__(kThreads) k_adamw_v4(const GT *__restrict__ g, float *__restrict__ V,
+                                                        int64_t rows, int64_t cols, float b2, float vcorr,
+                                                        float *__restrict__ colsum)
 {
     griddep_wait();
-    const int64_t c = 4 * ((int64_t)blockIdx.x * kCols + threadIdx.x);
-    const int64_t r0 = (int64_t)blockIdx.y * kRows1;
-    if (c >= cols)
-        return;
-    const int64_t r1 = r0 + kRows1 < rows ? r0 + kRows1 : rows;
+    const int64_t c = 4 * ((int64_t)blockIdx.x * kLanes + threadIdx.x % kLanes);
+    const int64_t r0 = ((int64_t)blockIdx.y * kGroups + threadIdx.x / kLanes) * kRows;
+    const int64_t r1 = c < cols ? (r0 + kRows < rows ? r0 + kRows : rows) : 0;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int64_t rb = r0; rb < r1; rb += kUnroll1) {
         float4 gv[kUnroll1], vv[kUnroll1];
@@ -153,6 +181,9 @@ __global__ void __launch_bounds__(kCols) k_adamw_v4(const GT *__restrict__ g, fl
                 s.w += v.w * vcorr;
             }
     }
+    s = sum_groups(s);
+    if (threadIdx.x >= kLanes || c >= cols)
+        return;
     atomicAdd(colsum + c, s.x);
     atomicAdd(colsum + c + 1, s.y);
     atomicAdd(colsum + c + 2, s.z);
@@ -211,14 +242,14 @@ template <typename GT>
 cudaError_t moments(const GT *g, float *M, float *V, int64_t rows, int64_t cols, float b1, float b2,
                     float vcorr, float *colsum, cudaStream_t s)
 {
+    const unsigned y = (unsigned)((rows + kGroups * kRows - 1) / (kGroups * kRows));
     count_launch();
     if (cols % 4 != 0)
         return launch_dependent(k_adamw_moments<GT>,
-                                dim3((unsigned)((cols + kCols - 1) / kCols), (unsigned)((rows + kRows - 1) / kRows)),
-                                dim3(kCols), 0, s, g, M, V, rows, cols, b1, b2, vcorr, colsum);
-    return launch_dependent(k_adamw_v4<GT>,
-                            dim3((unsigned)((cols / 4 + kCols - 1) / kCols), (unsigned)((rows + kRows1 - 1) / kRows1)),
-                            dim3(kCols), 0, s, g, V, rows, cols, b2, vcorr, colsum);
+                                dim3((unsigned)((cols + kLanes - 1) / kLanes), y), dim3(kThreads), 0, s, g, M,
+                                V, rows, cols, b1, b2, vcorr, colsum);
+    return launch_dependent(k_adamw_v4<GT>, dim3((unsigned)((cols / 4 + kLanes - 1) / kLanes), y),
+                            dim3(kThreads), 0, s, g, V, rows, cols, b2, vcorr, colsum);
 }
 
 // The second pass: W (and M)

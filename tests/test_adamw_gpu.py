@@ -106,3 +106,19 @@ def test_row_blocks(sn, rows, cols):
     sn.sn_adamw_rowconst(W, grad, M, V, 2, 1e-3, 0.9, 0.95, 1e-8, 1e-4)
     for got, want in ((W, W64), (M, M64), (V, V64)):
         assert float((got.double() - want).norm() / want.norm()) <= 1e-6
+
+
+@pytest.mark.parametrize("cols", [4, 3])
+def test_column_sums_take_one_addition_per_64_rows(sn, cols):
+    """Equal gradients down a column make every partial sum equal, so the sum's rounding does
+    not depend on the order of arrival.  n additions of equal terms to a running sum S err
+    by at most half an ulp of it each, n / 2 * 2^-24 of the final sum; 64 rows meet before
+    a column takes an addition.  With beta = 0, eps = 0, lr = 1 and W = 0 the step is
+    -g / sqrt(mean g^2) = -1, with half the sum's relative error."""
+    rows = 1 << 20
+    g = torch.tensor([1.922119140625, 1.453369140625, 1.312744140625, 1.218994140625][:cols])
+    grad = g.cuda().expand(rows, cols).contiguous()
+    W, M, V = (torch.zeros(rows, cols, device="cuda") for _ in range(3))
+    sn.sn_adamw_rowconst(W, grad, M, V, 1, 1.0, 0.0, 0.0, 0.0, 0.0)
+    bound = 0.5 * (rows / 64 / 2 + 64) * 2.0 ** -24 + 8 * 2.0 ** -24
+    assert float((W.double() + 1).abs().max()) <= bound
