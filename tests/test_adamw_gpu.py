@@ -122,3 +122,44 @@ def test_column_sums_take_one_addition_per_64_rows(sn, cols):
     sn.sn_adamw_rowconst(W, grad, M, V, 1, 1.0, 0.0, 0.0, 0.0, 0.0)
     bound = 0.5 * (rows / 64 / 2 + 64) * 2.0 ** -24 + 8 * 2.0 ** -24
     assert float((W.double() + 1).abs().max()) <= bound
+
+
+@pytest.mark.parametrize("gdt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("rows,cols", [(5000, 1), (4097, 2), (5, 3), (4096 + 1, 4), (2050, 5), (777, 8),
+                                       (1030, 12), (511, 33), (131, 63), (65, 65), (300, 252), (129, 260)])
+def test_narrow_weights(sn, gdt, rows, cols):
+    """Blocks with fewer lanes along the columns, at both sides of their row runs' ends: the
+    step against the definition in fp64, bars as in test_row_blocks."""
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    W, M, grad = (torch.randn(rows, cols, generator=g, device="cuda") for _ in range(3))
+    V = torch.rand(rows, cols, generator=g, device="cuda")
+    grad = grad.to(gdt)
+    M64 = 0.9 * M.double() + 0.1 * grad.double()
+    V64 = 0.95 * V.double() + 0.05 * grad.double() ** 2
+    rate = (V64.mean(0) / (1 - 0.95 ** 2)).sqrt() + 1e-8
+    W64 = W.double() - 1e-3 * (M64 / (1 - 0.9 ** 2)) / rate - 1e-4 * W.double()
+    sn.sn_adamw_rowconst(W, grad, M, V, 2, 1e-3, 0.9, 0.95, 1e-8, 1e-4)
+    for got, want in ((W, W64), (M, M64), (V, V64)):
+        assert float((got.double() - want).norm() / want.norm()) <= 1e-6
+
+
+@pytest.mark.parametrize("cols", [4, 1])
+def test_a_narrow_weight_costs_like_a_wide_one(sn, cols):
+    """As many elements in a few columns: every thread of a block has rows to work on, so the
+    step takes less than ten times as long as the same number of elements in 1024 columns
+    (a block with one busy thread in 256 takes thirty times as long)."""
+    def fastest(rows, cols):
+        W, grad, M, V = (torch.rand(rows, cols, device="cuda") for _ in range(4))
+        ws = torch.empty(4 * cols, dtype=torch.uint8, device="cuda")
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        times = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            ev[0].record()
+            for _ in range(4):
+                sn.sn_adamw_rowconst(W, grad, M, V, 2, 1e-3, workspace=ws)
+            ev[1].record()
+            ev[1].synchronize()
+            times.append(ev[0].elapsed_time(ev[1]))
+        return min(times)
+    assert fastest((1 << 22) // cols, cols) <= 10 * fastest(1 << 12, 1 << 10)
