@@ -600,9 +600,10 @@ cudaError_t grassmann_step(const sn_basis &b, const float *M, int K, float eta, 
         e = cudaMemsetAsync(p.bar, 0, 2 * sizeof(unsigned int), s);
     if (e != cudaSuccess)
         return e;
-    // cooperative: the CTAs wait for one another, so all are resident (one per SM)
+    // cooperative: the CTAs wait for one another, so all are resident, one on each SM
+    // that the stream's context has
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(std::min(p.nblk, sm_count()));
+    cfg.gridDim = dim3(std::min(p.nblk, stream_sms(s)));
     cfg.blockDim = dim3(kStepThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

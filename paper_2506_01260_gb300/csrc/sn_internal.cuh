@@ -138,6 +138,9 @@ cudaError_t simt_project(const sn_basis &b, const float *W, int64_t cols, int64_
                          float *A, cudaStream_t s);
 int simt_padded_columns(int k);   // sn_basis::kp
 
+// SMs available to kernels on a stream (fewer than the device's in a green context)
+int stream_sms(cudaStream_t s);
+
 cudaError_t prepare_basis(sn_basis &b, const float *U, cudaStream_t s);
 
 // ---- tensor-core kernels (bf16 path, tcgen05 + TMA) -----------------------------

@@ -674,4 +674,41 @@ cudaError_t tc_project(const sn_basis &b, const __nv_bfloat16 *W, int64_t cols, 
     return launch_expand(AMODE_TMA, q, std::min(q.ntiles * q.chunks, sms), s);
 }
 
+// The SMs that kernels launched on `s` may use: those of its context, which are fewer than
+// the device's in a green context, on its streams and wherever it is current.
+int stream_sms(cudaStream_t s)
+{
+    typedef CUresult (*StreamGetCtx)(CUstream, CUcontext *, CUgreenCtx *);
+    typedef CUresult (*CtxGetResource)(CUcontext, CUdevResource *, CUdevResourceType);
+    typedef CUresult (*GreenGetResource)(CUgreenCtx, CUdevResource *, CUdevResourceType);
+    static StreamGetCtx stream_ctx = nullptr;
+    static CtxGetResource ctx_resource = nullptr;
+    static GreenGetResource green_resource = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        auto find = [](const char *name, unsigned int version) {
+            void *f = nullptr;
+            cudaDriverEntryPointQueryResult q;
+            return cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &q) ==
+                               cudaSuccess &&
+                           q == cudaDriverEntryPointSuccess
+                       ? f
+                       : nullptr;
+        };
+        stream_ctx = (StreamGetCtx)find("cuStreamGetCtx", 12050);
+        ctx_resource = (CtxGetResource)find("cuCtxGetDevResource", 12040);
+        green_resource = (GreenGetResource)find("cuGreenCtxGetDevResource", 12040);
+    });
+    const int all = tc::sm_count(tc::current_device());
+    CUcontext ctx = nullptr;
+    CUgreenCtx green = nullptr;
+    CUdevResource r;
+    if (!stream_ctx || !ctx_resource || !green_resource ||
+        stream_ctx((CUstream)s, &ctx, &green) != CUDA_SUCCESS ||
+        (green ? green_resource(green, &r, CU_DEV_RESOURCE_TYPE_SM)
+               : ctx_resource(ctx, &r, CU_DEV_RESOURCE_TYPE_SM)) != CUDA_SUCCESS)
+        return all;
+    return std::max(1, std::min(all, (int)r.sm.smCount));
+}
+
 }  // namespace sn
