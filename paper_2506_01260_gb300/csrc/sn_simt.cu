@@ -97,15 +97,17 @@ __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
-// CTAs per cluster that share one output tile's reduction: the power of two up
+// CTAs per cluster that share one output tile's reduction: 1 where the stream's context
+// has not all of the SMs (a cluster might find no place in it), else the power of two up
 // to 8 with the least (rounds of the grid) x (steps per CTA + 3 for its start + one
 // for each CTA whose partial sums meet), every CTA keeping at least one step.  Among
 // equal costs, the fewest CTAs.  Measured on whole calls, with 1 / 2 / 4 / 8 CTAs (W one
 // step ahead): projection of [2048, 2048] at k = 20 (16 tiles) 74 / 48 / 33 / 37 us, of
 // [2048, 8192] (64 tiles) 92 / 67 / 72 / 90 us; compress of 8192 x 2048 (256 tiles) 31 /
 // 34 / 35 / 43 us.
-int cluster_split(int64_t tiles, int steps, int64_t slots)
+int cluster_split(int64_t tiles, int steps, int sms, int per_sm, cudaStream_t s)
 {
+    const int64_t slots = (int64_t)sms * per_sm;
     int best = 1;
     int64_t best_cost = -1;
     for (int c = 1; c <= 8 && c <= steps; c *= 2) {
@@ -116,7 +118,7 @@ int cluster_split(int64_t tiles, int steps, int64_t slots)
             best = c;
         }
     }
-    return best;
+    return best > 1 && stream_sms(s) < sms ? 1 : best;
 }
 
 // ---- C[t, :] = (X[t, :] - tok[id] - pe[p]) U  (or G U when !GATHER) -----------
@@ -695,7 +697,7 @@ cudaError_t launch_compress_f32(SimtCompress p, bool gather, int sms, cudaStream
     const int64_t tiles = (p.T + CTOK - 1) / CTOK;
     const int steps = ((p.d + CCH - 1) / CCH + G - 1) / G;
     // registers let two (gather) or three CTAs share an SM
-    p.split = cluster_split(tiles, steps, (int64_t)sms * (gather ? 2 : 3));
+    p.split = cluster_split(tiles, steps, sms, gather ? 2 : 3, s);
     const unsigned grid = (unsigned)(tiles * p.split);
     void (*const kernel)(SimtCompress) =
         gather ? k_simt_compress<WN, TN, true> : k_simt_compress<WN, TN, false>;
@@ -741,7 +743,7 @@ cudaError_t launch_project_a(SimtProject p, int sms, cudaStream_t s)
     constexpr size_t red = sizeof(float) * G * KP * 128;
     const int64_t tiles = (p.cols + 127) / 128;
     const int steps = (p.d + PROWS * G - 1) / (PROWS * G);
-    p.split = cluster_split(tiles, steps, sms);
+    p.split = cluster_split(tiles, steps, sms, 1, s);
     constexpr size_t smem = stage > red ? stage : red;
     cudaError_t e = cudaFuncSetAttribute(k_simt_project_a<WN, JT>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -2,7 +2,9 @@
 
 The Grassmann step's CTAs wait for one another, so its grid may be no larger than the SMs
 that the stream's context has; with fewer a CTA owns several blocks of rows.  Bars as for
-the step on the whole GPU."""
+the step on the whole GPU.  The fp32 calls share a reduction among the CTAs of a cluster,
+which such a context may have no place for: there they run without clusters.  Their bars:
+d fp32 products summed in any order, d * 2^-24 of the sum of magnitudes."""
 import ctypes
 
 import numpy as np
@@ -76,4 +78,30 @@ def test_step_on_part_of_the_sms(sn, green, d, k):
     got = out.cpu().numpy().astype(np.float64)
     assert rel(got, o.step(U32.astype(np.float64), M32.astype(np.float64), 1, eta)) <= 1e-4
     assert np.max(np.abs(got.T @ got - np.eye(k))) <= 1e-5
+    basis.destroy()
+
+
+def test_fp32_reductions_on_part_of_the_sms(sn, green):
+    T, d, k, cols = 40, 2048, 20, 200                      # a few tiles: clusters on the whole GPU
+    g = torch.Generator().manual_seed(5)
+    U = torch.linalg.qr(torch.randn(d, k, generator=g, dtype=torch.float64))[0].float().contiguous().cuda()
+    X, Wt = torch.randn(T, d, generator=g).cuda(), torch.randn(d, cols, generator=g).cuda()
+    tok, ids = torch.randn(50, d, generator=g).cuda(), torch.randint(50, (T,), generator=g).int().cuda()
+    basis = sn.Basis(U)
+    Cf, Cb, Wo = torch.empty(T, k, device="cuda"), torch.empty(T, k, device="cuda"), torch.empty_like(Wt)
+    ws = torch.empty(sn.sn_project_weight_workspace(basis, torch.float32, cols), dtype=torch.uint8,
+                     device="cuda")
+    torch.cuda.synchronize()
+    s = green.stream.value
+    sn.sn_compress_fwd(basis, X, ids, tok, T, out=Cf, stream=s)
+    sn.sn_compress_bwd(basis, X, out=Cb, stream=s)
+    sn.sn_project_weight(basis, Wt, out=Wo, workspace=ws, stream=s)
+    green.synchronize()
+    sn.sn_check_errors(basis)
+    U64, W64, R64 = U.double(), Wt.double(), X.double() - tok[ids.long()].double()
+    A = U64.abs().T @ W64.abs()
+    for got, want, size in ((Cb, X.double() @ U64, X.double().abs() @ U64.abs()),
+                            (Cf, R64 @ U64, (R64.abs() + X.double().abs()) @ U64.abs()),
+                            (Wo, U64 @ (U64.T @ W64), 2 * U64.abs() @ A)):
+        assert ((got.double() - want).abs() <= d * 2.0 ** -24 * size).all()
     basis.destroy()
