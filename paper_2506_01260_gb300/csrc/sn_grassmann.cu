@@ -181,7 +181,8 @@ __device__ __forceinline__ void two_sum(float &s, float &e, float v)
 // This CTA's slice of out[e] = sum over the blocks of part[blk, e]: 32 elements a warp,
 // the warps that are left over sharing out the blocks.  The sums carry their
 // rounding errors along (Knuth's two-sum), so they are as good as fp64 ones rounded
-// once; a chain of fp64 additions took 3 us a slice on this GPU.
+// once; a chain of fp64 additions took 3 us a slice on this GPU.  Where fp32 overflows, the
+// pair says nothing and the element is summed again in fp64.
 __device__ __noinline__ void sum_slice(const StepParams &p, float *out, float2 *red)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -212,7 +213,14 @@ __device__ __noinline__ void sum_slice(const StepParams &p, float *out, float2 *
                 two_sum(s, err, v.x);
                 err += v.y;
             }
-            out[e0 + e] = s + err;
+            s += err;
+            if (!isfinite(s)) {
+                double t = 0.0;
+                for (int b = 0; b < p.nblk; ++b)
+                    t += (double)__ldcg(p.part + (size_t)b * kk + e0 + e);
+                s = (float)t;
+            }
+            out[e0 + e] = s;
         }
         __syncthreads();
     }

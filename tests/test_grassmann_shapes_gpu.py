@@ -55,3 +55,23 @@ def test_accumulate_shapes(sn, d, k, T):
     assert rel(M.cpu().numpy().astype(np.float64), g.accumulate(np.zeros((d, k)), G64, U64)) <= 1e-2
     assert abs(acc.item() - g.residual(G64, U64)) <= 1e-3 * np.sum(G64 * G64)
     basis.destroy()
+
+
+@pytest.mark.parametrize("signs", [(1, 1, -1, -1), (1, -1, 1, -1)])
+def test_step_sums_past_fp32(sn, signs):
+    """Block sums of U^T M near fp32's largest number, two of either sign: on the way the sum
+    passes what fp32 holds, and is 0 in the end.  The step moves U by about 24 times its
+    norm; bars as above."""
+    g = grassmann_oracle()
+    d, eta = 256, 1e-38
+    U32 = np.full((d, 1), 1 / 16, np.float32)
+    M32 = np.repeat(np.float32(7.5e37) * np.array(signs, np.float32), 64).reshape(d, 1)
+    basis = sn.Basis(dev(U32))
+    got = sn.sn_grassmann_step(basis, dev(M32), 1, eta)
+    sn.sn_check_errors(basis)
+    got = got.cpu().numpy().astype(np.float64)
+    # the step size reaches the kernel as 2 eta rounded to fp32
+    ref = g.step(U32.astype(np.float64), M32.astype(np.float64), 1, float(np.float32(2 * np.float32(eta))) / 2)
+    assert rel(got, ref) <= 1e-4
+    assert abs((got.T @ got).item() - 1) <= 1e-5
+    basis.destroy()
