@@ -491,10 +491,11 @@ __global__ void __launch_bounds__(256) k_transpose_pad(const __nv_bfloat16 *__re
 {
     // 64 tokens per block through shared memory: a warp reads eight k-wide rows
     // (adjacent, so coalesced; all eight in flight), each output row j gets 64
-    // consecutive tokens (128-byte writes, two tokens a thread); the row pitch of 130
-    // elements keeps the column reads on distinct banks.  k <= 128.  3.8 us for 16384
+    // consecutive tokens (128-byte writes, two tokens a thread); the row pitch of 129
+    // elements puts a lane's row pair 129 words from its neighbour's, so that the column
+    // reads fall in distinct banks.  k <= 128.  3.8 us for 16384
     // tokens at k = 41 (10 us with a division per element).
-    __shared__ __nv_bfloat16 tile[64][130];
+    __shared__ __nv_bfloat16 tile[64][129];
     griddep_wait();
     const int64_t t0 = (int64_t)blockIdx.x * 64;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
