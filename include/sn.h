@@ -316,6 +316,11 @@ sn_status sn_check_errors(sn_basis_t basis, sn_stream_t stream);
  * another device), SN_ERR_CUDA (launch failure). */
 sn_status sn_selftest_wait_timeout(sn_basis_t basis, sn_stream_t stream);
 
+/* The same for the grid barrier in which the CTAs of sn_grassmann_step wait for one
+ * another: one CTA waits for arrivals that nobody makes, gives up at the limit with
+ * SN_ERR_TIMEOUT, and a second wait ends at once on the flag that the first one left. */
+sn_status sn_selftest_barrier_timeout(sn_basis_t basis, sn_stream_t stream);
+
 /* Number of kernels this library has launched in this process. */
 uint64_t sn_launch_count(void);
 

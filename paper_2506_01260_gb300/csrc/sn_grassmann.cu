@@ -51,38 +51,6 @@ struct StepParams {
     float beta, gamma;          // A = U + beta M + gamma U Y
 };
 
-// Every CTA of the grid has arrived `n` times: their writes before it are visible
-// (through L2: read them with __ldcg).  Bounded like every wait of the library; false
-// when it gave up, in which case every CTA leaves.
-__device__ __noinline__ bool grid_barrier(const StepParams &p, unsigned int n)
-{
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(p.bar, 1u);
-        const uint64_t t0 = tc::global_ns();
-        volatile unsigned int *bar = p.bar;
-        int o = 1;
-        while (bar[0] < n * gridDim.x) {
-            if (bar[1]) {
-                o = 0;
-                break;
-            }
-            if (tc::global_ns() - t0 > tc::kWaitLimitNs) {
-                bar[1] = 1u;
-                atomicOr(p.err, SN_EBIT_TIMEOUT);
-                o = 0;
-                break;
-            }
-        }
-        __threadfence();
-        ok = o;
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
 // dst[r][c] = src[row0 + r, c] for the block's rows, zero past d and k (pitch k4 <=
 // 128).  A warp takes four rows, all its loads in flight before the first store.
 __device__ __forceinline__ void load_rows(float *dst, const float *src, int row0, int d, int k, int k4)
@@ -422,10 +390,10 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_grassmann_step(StepParams p
     const bool one = p.nblk <= (int)gridDim.x;       // a block of rows per CTA, kept in sa
     unsigned int nbar = 0;
     auto reduce = [&](float *out) {                  // out = the sum of all partial products
-        if (!grid_barrier(p, ++nbar))
+        if (!tc::grid_barrier(p.bar, ++nbar, p.err))
             return false;
         sum_slice(p, out, (float2 *)red);
-        return grid_barrier(p, ++nbar);
+        return tc::grid_barrier(p.bar, ++nbar, p.err);
     };
     // Y = U^T M
     for (int blk = blockIdx.x; blk < p.nblk; blk += gridDim.x) {

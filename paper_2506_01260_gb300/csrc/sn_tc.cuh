@@ -187,6 +187,40 @@ __device__ __forceinline__ void drain_wait(uint32_t bar, uint32_t parity)
     }
 }
 
+// ---- grid barrier (cooperative launches) --------------------------------------------
+// Every CTA of the grid has arrived `n` times: their writes before it are visible
+// (through L2: read them with __ldcg).  `bar`: the arrivals, and a flag that a wait gave
+// up, both zeroed before the launch.  Bounded like every wait of the library; false when
+// it gave up, in which case every CTA leaves.
+[[maybe_unused]] static __device__ __noinline__ bool grid_barrier(unsigned int *bar, unsigned int n, unsigned int *err)
+{
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        const uint64_t t0 = global_ns();
+        volatile unsigned int *b = bar;
+        int o = 1;
+        while (b[0] < n * gridDim.x) {
+            if (b[1]) {
+                o = 0;
+                break;
+            }
+            if (global_ns() - t0 > kWaitLimitNs) {
+                b[1] = 1u;
+                atomicOr(err, SN_EBIT_TIMEOUT);
+                o = 0;
+                break;
+            }
+        }
+        __threadfence();
+        ok = o;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 // ---- TMA ---------------------------------------------------------------------------
 __device__ __forceinline__ void tma_prefetch(const CUtensorMap *m)
 {

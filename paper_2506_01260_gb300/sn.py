@@ -70,6 +70,7 @@ _sig("sn_wire_send", [_P, _P, _SZ, _P])
 _sig("sn_wire_recv", [_P, _P, _SZ, _P])
 _sig("sn_check_errors", [_P, _P])
 _sig("sn_selftest_wait_timeout", [_P, _P])
+_sig("sn_selftest_barrier_timeout", [_P, _P])
 _sig("sn_launch_count", [], ctypes.c_uint64)
 _sig("sn_status_string", [_ST], ctypes.c_char_p)
 
@@ -82,7 +83,8 @@ EXPORTS = ["sn_basis_create", "sn_basis_destroy", "sn_basis_shape", "sn_compress
            "sn_grassmann_step", "sn_adamw_rowconst", "sn_topk_compress", "sn_topk_restore",
            "sn_sign_compress", "sn_sign_restore", "sn_quant_compress", "sn_quant_restore",
            "sn_wire_bytes", "sn_wire_send",
-           "sn_wire_recv", "sn_check_errors", "sn_selftest_wait_timeout", "sn_launch_count",
+           "sn_wire_recv", "sn_check_errors", "sn_selftest_wait_timeout",
+           "sn_selftest_barrier_timeout", "sn_launch_count",
            "sn_status_string"]
 
 
@@ -614,6 +616,13 @@ def sn_selftest_wait_timeout(basis, stream=None):
     SN_ERR_TIMEOUT for the next sn_check_errors."""
     _check(_lib.sn_selftest_wait_timeout(basis.handle, _stream(stream)),
            "sn_selftest_wait_timeout")
+
+
+def sn_selftest_barrier_timeout(basis, stream=None):
+    """The same for the grid barrier of sn_grassmann_step: one CTA waits for arrivals that
+    nobody makes and gives up at the limit."""
+    _check(_lib.sn_selftest_barrier_timeout(basis.handle, _stream(stream)),
+           "sn_selftest_barrier_timeout")
 
 
 def sn_launch_count():

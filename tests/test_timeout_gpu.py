@@ -54,3 +54,35 @@ def test_selftest_rejects_bad_arguments(sn):
     with pytest.raises(sn.SNError) as e:
         sn.sn_selftest_wait_timeout(Null())
     assert e.value.status == sn.SN_ERR_INVALID_ARG
+
+
+def test_expired_grid_barrier_reports_timeout_and_the_step_runs_after_it(sn):
+    d, k = 1024, 20
+    g = torch.Generator().manual_seed(4)
+    U = torch.linalg.qr(torch.randn(d, k, generator=g, dtype=torch.float64))[0].float().contiguous().cuda()
+    M = torch.randn(d, k, generator=g).cuda()
+    basis = sn.Basis(U)
+    before = sn.sn_grassmann_step(basis, M, 1, 1e-3)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    a.record()
+    sn.sn_selftest_barrier_timeout(basis)
+    b.record()
+    with pytest.raises(sn.SNError) as e:
+        sn.sn_check_errors(basis)
+    assert e.value.status == sn.SN_ERR_TIMEOUT
+    # the first wait lasts as long as the limit, the second ends on the flag it left
+    elapsed = a.elapsed_time(b) / 1e3
+    assert LIMIT_S * 0.95 <= elapsed <= LIMIT_S * 1.5, elapsed
+    after = sn.sn_grassmann_step(basis, M, 1, 1e-3)
+    sn.sn_check_errors(basis)                 # reported once, and the step is as before
+    assert torch.equal(before, after)
+    basis.destroy()
+
+
+def test_barrier_selftest_rejects_bad_arguments(sn):
+    class Null:
+        handle = None
+    with pytest.raises(sn.SNError) as e:
+        sn.sn_selftest_barrier_timeout(Null())
+    assert e.value.status == sn.SN_ERR_INVALID_ARG
