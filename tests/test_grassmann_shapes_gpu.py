@@ -75,3 +75,30 @@ def test_step_sums_past_fp32(sn, signs):
     assert rel(got, ref) <= 1e-4
     assert abs((got.T @ got).item() - 1) <= 1e-5
     basis.destroy()
+
+
+@pytest.mark.parametrize("d,k,T", [(128, 7, 1), (256, 33, 63), (264, 64, 65), (512, 127, 129),
+                                   (136, 2, 20000)])
+def test_accumulate_and_residual_of_what_the_kernels_read(sn, d, k, T):
+    """G^T Cg and |G|^2 - |Cg|^2 in fp64 from the bf16 G and Cg themselves.  M: products exact in
+    fp32, an addition for every 16 tokens and split, each off by at most an ulp of a sum no
+    larger than the last.  The residual: runs of 128 squares in fp32, off by about
+    sqrt(128) / 2 * 2^-24 = 3.4e-7 of themselves at random, the rest in fp64.  Both bars lie below
+    what one lost token, or one lost 16-byte piece of G, makes."""
+    U32, (Gb,) = basis_and_grads(sn, d, k, T, 1, seed=T + k)
+    basis = sn.Basis(dev(U32))
+    G = dev(Gb)
+    Cg = sn.sn_compress_bwd(basis, G)
+    M0 = torch.full((d, k), 0.5, device="cuda")
+    M, acc = M0.clone(), torch.full((1,), 3.0, dtype=torch.float64, device="cuda")
+    sn.sn_grassmann_accumulate(basis, G, Cg, M)
+    sn.sn_grassmann_residual(basis, G, Cg, acc)
+    sn.sn_check_errors(basis)
+    G64, C64 = G.double(), Cg.double()
+    want, sq = M0.double() + G64.T @ C64, G64.square().sum().item()
+    m_bar, r_bar = (T / 16 + 16) * 2.0 ** -23 * want.norm().item(), 1e-6 * (sq + C64.square().sum().item())
+    assert (M.double() - want).norm().item() <= m_bar
+    assert abs(acc.item() - 3.0 - (sq - C64.square().sum().item())) <= r_bar
+    lost = min((G64[t].norm() * C64[t].norm()).item() for t in (0, T // 2, T - 1))
+    assert m_bar < lost and r_bar < G64[-1, -8:].square().sum().item()
+    basis.destroy()
