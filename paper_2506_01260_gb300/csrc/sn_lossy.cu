@@ -216,13 +216,15 @@ __global__ void __launch_bounds__(kThreads) k_topk(const uint16_t *__restrict__ 
         int bound = -1;
         if (M > 0 && q <= 32) {
             // (the lanes' values agree above their first differing bit, and a bound
-            // up to 3 keys low only admits a few more candidates)
+            // up to 3 keys low only admits a few more candidates; for M = 4, where those
+            // few can be more than a warp holds, it is searched to the last bit: T = 16384,
+            // d = 4096, kk = 96 took 81 us with the low bound, now 53)
             const int vl = top[M > 0 ? M - 1 : 0];
             const int hi = max(__reduce_max_sync(0xffffffffu, vl), 0);
             const int lo = max(__reduce_min_sync(0xffffffffu, vl), 0);
             int bit = 31 - __clz(lo ^ hi);
             int b = hi & ~((1 << (bit + 1)) - 1);
-            for (; bit >= 2; --bit)
+            for (; bit >= (M < 4 ? 2 : 0); --bit)
                 if (warp_count(vl >= (b | (1 << bit))) >= q)
                     b |= 1 << bit;
             bound = warp_count(vl >= b) >= q ? b : -1;
@@ -273,21 +275,30 @@ __global__ void __launch_bounds__(kThreads) k_topk(const uint16_t *__restrict__ 
         // every entry at or above the bound is a candidate, so for any trial
         // the candidate count decides "at least kk entries reach it" as the
         // whole row would
-        // (the first 64 candidates' keys stay in registers; thr lies between the
-        // bound and the row's largest key, so their common bits are not searched:
-        // with the same shortcut for the bound above, T = 16384, d = 4096, kk = 20
-        // took 48 -> 40 us)
-        const int key0 = lane < nc ? (int)(cand[lane] & 0x7FFFu) : -1;
-        const int key1 = lane + 32 < nc ? (int)(cand[lane + 32] & 0x7FFFu) : -1;
+        // (the candidates' keys stay in registers; thr lies between the bound and the row's
+        // largest key, so their common bits are not searched.  T = 16384, d = 4096, kk = 20:
+        // 45 -> 33 us with the same shortcut for the bound above.  Up to 64 candidates
+        // two votes count them, past that the lanes' own counts and one sum: with a vote
+        // per 32 candidates read from shared memory, T = 30000, d = 1024, kk = 64 took 82
+        // us instead of 63)
+        constexpr int kKeys = kWCap / 32;
+        int key[kKeys];
+#pragma unroll
+        for (int i = 0; i < kKeys; ++i)
+            key[i] = lane + 32 * i < nc ? (int)(cand[lane + 32 * i] & 0x7FFFu) : -1;
         auto reach = [&](int trial) {
-            int cnt = warp_count(key0 >= trial) + warp_count(key1 >= trial);
-            for (int j = 64 + lane; j < nc + lane; j += 32)               // warp-uniform
-                cnt += warp_count(j < nc && (int)(cand[j] & 0x7FFFu) >= trial);
-            return cnt;
+            if (nc <= 64)                                                  // warp-uniform
+                return warp_count(key[0] >= trial) + warp_count(key[1] >= trial);
+            int cnt = 0;
+#pragma unroll
+            for (int i = 0; i < kKeys; ++i)
+                cnt += key[i] >= trial;
+            return (int)__reduce_add_sync(0xffffffffu, cnt);
         };
-        int rmax = max(key0, key1);
-        for (int j = 64 + lane; j < nc; j += 32)
-            rmax = max(rmax, (int)(cand[j] & 0x7FFFu));
+        int rmax = key[0];
+#pragma unroll
+        for (int i = 1; i < kKeys; ++i)
+            rmax = max(rmax, key[i]);
         rmax = __reduce_max_sync(0xffffffffu, rmax);
         int bit = 31 - __clz(rmax ^ max(bound, 0));
         int thr = rmax & ~((1 << (bit + 1)) - 1);
