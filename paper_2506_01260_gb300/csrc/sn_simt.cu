@@ -520,6 +520,59 @@ __global__ void __launch_bounds__(ETHREADS, 2) k_simt_expand(const SimtExpand p)
     }
 }
 
+// The same for few rows: a thread owns one column and 8 rows and reads its column of R from
+// L2, so that a CTA starts without a copy of R and a small output is spread over eight times
+// as many threads.  Bound by that chain of loads, eight in flight.  The sums' chains are the
+// same, and so are the bits.  65 rows, d = 1000, k = 128: 9.4 us without and 11.4 us with
+// embeddings, by the tile kernel 15.9 and 24.7; 1024 rows (512 CTAs) 15.2 and 17.2 against
+// 17.1 and 26.0; 2048 rows (1024 CTAs) 29.9 and 33.4 against 17.2 and 26.2.
+constexpr int FROWS = 8;        // rows per CTA
+constexpr int FTHREADS = 256;   // columns per CTA
+constexpr int FK = 128;         // largest k
+static_assert(FTHREADS / 32 == FROWS, "a warp copies a row");
+
+template <bool EMB>
+__global__ void __launch_bounds__(FTHREADS) k_simt_expand_few(const SimtExpand p)
+{
+    __shared__ __align__(16) float ls[FROWS][FK];
+    __shared__ int64_t rtok[FROWS], rpe[FROWS];
+    __shared__ int rstate[FROWS];
+    const int tid = threadIdx.x;
+    const int64_t c = (int64_t)blockIdx.x * FTHREADS + tid, r0 = (int64_t)blockIdx.y * FROWS;
+    const bool has_pe = EMB && p.pe != nullptr;
+    griddep_wait();
+    if (tid < FROWS)
+        rstate[tid] = token_rows(r0 + tid, p.rows, EMB, p.ids, p.pos, p.seq_len, p.vocab, has_pe,
+                                 (int)p.cols, &rtok[tid], &rpe[tid], p.err);
+    for (int j = tid & 31; j < p.k; j += 32) {       // a row per warp
+        const int m = tid >> 5;
+        ls[m][j] = r0 + m < p.rows ? p.L[(r0 + m) * p.k + j] : 0.f;
+    }
+    __syncthreads();
+    if (c >= p.cols)
+        return;
+    float acc[FROWS] = {};
+#pragma unroll 8
+    for (int j = 0; j < p.k; ++j) {
+        const float u = __ldg(p.R + (int64_t)j * p.ldr + c);
+#pragma unroll
+        for (int m = 0; m < FROWS; ++m)
+            acc[m] = fmaf(ls[m][j], u, acc[m]);
+    }
+#pragma unroll
+    for (int m = 0; m < FROWS; ++m) {
+        if (rstate[m] == ROW_SKIP)
+            continue;
+        float v = acc[m];
+        if (EMB && rstate[m] == ROW_OK) {
+            if (has_pe)
+                v += __ldg(p.pe + rpe[m] + c);
+            v += __ldg(p.tok + rtok[m] + c);
+        }
+        p.out[(r0 + m) * p.ldo + c] = rstate[m] == ROW_OK ? v : 0.f;
+    }
+}
+
 // ---- A = U^T W (fp32 [k, cols]), the projection's first pass ---------------------
 // A warp owns 128 columns of W (a thread four, as two pairs) and JT columns of U;
 // WN warps form a group that covers all k, and the groups of a CTA and the CTAs of
@@ -735,6 +788,15 @@ cudaError_t launch_expand_f32(const SimtExpand &p, int sms, cudaStream_t s)
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+template <bool EMB>
+cudaError_t launch_expand_few(const SimtExpand &p, cudaStream_t s)
+{
+    const dim3 grid((unsigned)((p.cols + FTHREADS - 1) / FTHREADS), (unsigned)((p.rows + FROWS - 1) / FROWS));
+    const cudaError_t e = launch_dependent(k_simt_expand_few<EMB>, grid, dim3(FTHREADS), 0, s, p);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int WN, int JT>
 cudaError_t launch_project_a(SimtProject p, int sms, cudaStream_t s)
 {
@@ -752,6 +814,26 @@ cudaError_t launch_project_a(SimtProject p, int sms, cudaStream_t s)
                             dim3(PTHREADS), smem, s, p);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// Where the kernel for few rows is the faster one.  Five of its CTAs fit an SM.  Without
+// embeddings, as long as all are there at once (counted by their columns, four an SM: they
+// are bound by their FMAs then): 1024 rows of d = 1000, k = 41 take 6.9 us, 9.4 with tiles;
+// 2048 rows 11.8 and 9.5.  With embeddings the tile kernel takes its 128 columns in two
+// halves and runs in rounds: of one tile an SM while there are no more, in the time of one
+// round of the other's CTAs; else of two tiles an SM, in the time of 1.8 (2.05 for k > 32); for
+// k > 72, whose shared memory leaves no room for a second tile, of one, in 1.3.  6001 rows
+// of d = 1000, k = 41 take 33.7 us and 37.7 with tiles (3004 CTAs, two rounds), 2048 rows
+// 16.4 and 15.1; 12000 rows of d = 200, k = 128 32.9 and 49.2, 2048 of 1000 33.4 and 26.1.
+bool few_rows(const SimtExpand &p, bool emb, int sms)
+{
+    const int64_t ctas = (p.cols + FTHREADS - 1) / FTHREADS * ((p.rows + FROWS - 1) / FROWS);
+    if (!emb)
+        return ctas <= 5 * (int64_t)sms && std::min<int64_t>(p.cols, FTHREADS) * ctas <= 4 * FTHREADS * (int64_t)sms;
+    const int64_t tiles = (p.cols + ETILE - 1) / ETILE * ((p.rows + ETILE - 1) / ETILE);
+    const int64_t slots = p.k > 72 ? sms : 2 * sms, rounds = (tiles + slots - 1) / slots;
+    const int64_t percent = tiles <= sms ? 100 : (p.k > 72 ? 130 : p.k > 32 ? 205 : 180) * rounds;
+    return 100 * ctas <= 5 * sms * percent && (p.rows + FROWS - 1) / FROWS <= 65535;
 }
 
 int sm_count_f32(int device)
@@ -800,6 +882,8 @@ cudaError_t simt_decompress(const sn_basis &b, const float *C, const int32_t *id
 {
     const SimtExpand p{C, b.u32t, tok, pe, ids, pos, X, b.err, T, b.d, b.d, b.d, vocab, b.k, seq_len};
     const int sms = sm_count_f32(b.device);
+    if (few_rows(p, gather, sms))
+        return gather ? launch_expand_few<true>(p, s) : launch_expand_few<false>(p, s);
     return gather ? launch_expand_f32<true>(p, sms, s) : launch_expand_f32<false>(p, sms, s);
 }
 

@@ -10,6 +10,7 @@ is a missing or doubled product's, not the arithmetic's.
 """
 import numpy as np
 import pytest
+import torch
 
 from gpu_util import assert_parity, dev, guarded, guards_intact, host
 from paper_2506_01260_gb300 import workloads as W
@@ -67,3 +68,58 @@ def test_f32_projection_shapes(sn, oracle, d, k, cols, pad):
     _, W64, _ = oracle.project_weight(np.ascontiguousarray(Wh[:, :cols]), U)
     assert_parity(host(out[:, :cols]), W64, "f32")
     basis.destroy()
+
+
+@pytest.mark.parametrize("d,k", [(16, 1), (264, 5), (520, 20), (1000, 41), (136, 64), (2056, 127), (512, 128)])
+@pytest.mark.parametrize("with_pos", [False, True])
+def test_few_rows_give_the_tiles_bits(sn, d, k, with_pos):
+    """Reconstruction of 4903 rows takes the tile kernel, of a few of them the one for few rows:
+    one chain of sums over j in both, so the same bits; ids out of range included."""
+    T, vocab, n = 4903, 50, 64
+    g = torch.Generator().manual_seed(d + k)
+    U = torch.linalg.qr(torch.randn(d, k, generator=g, dtype=torch.float64))[0].float().contiguous().cuda()
+    C, tok, pe = (torch.randn(r, w, generator=g).cuda() for r, w in ((T, k), (vocab, d), (n, d)))
+    ids = torch.randint(vocab, (T,), generator=g).int()
+    pos = torch.randint(n, (T,), generator=g).int()
+    ids[5], ids[4096], pos[9] = vocab, -1, n
+    ids, pos = ids.cuda(), pos.cuda()
+    basis = sn.Basis(U)
+
+    def both(t0, t1):
+        fwd = sn.sn_decompress_fwd(basis, C[t0:t1].clone(), ids[t0:t1].clone(), tok, n,
+                                   pos_emb=pe if with_pos else None,
+                                   pos=pos[t0:t1].clone() if with_pos else None)
+        return fwd, sn.sn_decompress_bwd(basis, C[t0:t1].clone())
+    whole = both(0, T)
+    for t0, rows in ((0, 1), (3, 7), (0, 8), (4090, 9), (100, 16), (1000, 130), (4803, 100)):
+        for w, f in zip(whole, both(t0, t0 + rows)):
+            assert torch.equal(f, w[t0:t0 + rows])
+    assert not whole[0][5].any() and not whole[0][4096].any() and bool(whole[0][6].any())
+    with pytest.raises(sn.SNError):
+        sn.sn_check_errors(basis)
+    basis.destroy()
+
+
+def test_few_rows_at_a_wide_basis_start_at_once(sn):
+    """65 rows at k = 128 read sixteen times the coefficients of k = 8 but take less than twice as
+    long (three times, where every CTA first copies 128 columns of U^T)."""
+    T, d = 65, 1000
+    tok = torch.randn(50, d, device="cuda")
+    ids = torch.randint(50, (T,), device="cuda", dtype=torch.int32)
+
+    def fastest(k):
+        U = torch.linalg.qr(torch.randn(d, k, dtype=torch.float64))[0].float().contiguous().cuda()
+        basis, C, out = sn.Basis(U), torch.randn(T, k, device="cuda"), torch.empty(T, d, device="cuda")
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        times = []
+        for _ in range(8):
+            torch.cuda.synchronize()
+            ev[0].record()
+            for _ in range(20):
+                sn.sn_decompress_fwd(basis, C, ids, tok, T, out=out)
+            ev[1].record()
+            ev[1].synchronize()
+            times.append(ev[0].elapsed_time(ev[1]))
+        basis.destroy()
+        return min(times)
+    assert fastest(128) <= 2 * fastest(8)
