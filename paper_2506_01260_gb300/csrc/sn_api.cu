@@ -198,8 +198,8 @@ sn_status sn_compress_fwd(sn_basis_t b, sn_dtype dt, const void *X, const int32_
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
         return cuda_status(sn::simt_compress(*b, (const float *)X, ids, pos, T, seq_len,
-                                                    (const float *)tok, vocab, (const float *)pe,
-                                                    (float *)C, true, s));
+                                             (const float *)tok, vocab, (const float *)pe,
+                                             (float *)C, true, s));
     sn::TcArgs a{(const __nv_bfloat16 *)X, ids, pos, (const __nv_bfloat16 *)tok,
                  (const __nv_bfloat16 *)pe, (__nv_bfloat16 *)C, T, vocab, seq_len, true};
     return cuda_status(sn::tc_compress(*b, a, s));
@@ -216,8 +216,8 @@ sn_status sn_decompress_fwd(sn_basis_t b, sn_dtype dt, const void *C, const int3
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
         return cuda_status(sn::simt_decompress(*b, (const float *)C, ids, pos, T, seq_len,
-                                                      (const float *)tok, vocab,
-                                                      (const float *)pe, (float *)X, true, s));
+                                               (const float *)tok, vocab,
+                                               (const float *)pe, (float *)X, true, s));
     sn::TcArgs a{nullptr, ids, pos, (const __nv_bfloat16 *)tok, (const __nv_bfloat16 *)pe,
                  (__nv_bfloat16 *)C, T, vocab, seq_len, true};
     return cuda_status(sn::tc_decompress(*b, a, (__nv_bfloat16 *)X, s));
@@ -243,7 +243,7 @@ sn_status sn_compress_bwd(sn_basis_t b, sn_dtype dt, const void *G, int64_t T, v
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
         return cuda_status(sn::simt_compress(*b, (const float *)G, nullptr, nullptr, T, 1,
-                                                    nullptr, 1, nullptr, (float *)C, false, s));
+                                             nullptr, 1, nullptr, (float *)C, false, s));
     sn::TcArgs a{(const __nv_bfloat16 *)G, nullptr, nullptr, nullptr, nullptr,
                  (__nv_bfloat16 *)C, T, 1, 1, false};
     return cuda_status(sn::tc_compress(*b, a, s));
@@ -269,8 +269,8 @@ sn_status sn_decompress_bwd(sn_basis_t b, sn_dtype dt, const void *C, int64_t T,
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
         return cuda_status(sn::simt_decompress(*b, (const float *)C, nullptr, nullptr, T,
-                                                      1, nullptr, 1, nullptr, (float *)G, false,
-                                                      s));
+                                               1, nullptr, 1, nullptr, (float *)G, false,
+                                               s));
     sn::TcArgs a{nullptr, nullptr, nullptr, nullptr, nullptr, (__nv_bfloat16 *)C, T, 1, 1,
                  false};
     return cuda_status(sn::tc_decompress(*b, a, (__nv_bfloat16 *)G, s));
@@ -320,7 +320,7 @@ sn_status sn_project_weight(sn_basis_t b, sn_dtype dt, const void *W, int64_t ro
     cudaStream_t s = (cudaStream_t)stream;
     if (dt == SN_F32)
         return cuda_status(sn::simt_project(*b, (const float *)W, cols, ld, (float *)W_out,
-                                                   (float *)ws, s));
+                                            (float *)ws, s));
     return cuda_status(sn::tc_project(*b, (const __nv_bfloat16 *)W, cols, ld,
                                       (__nv_bfloat16 *)W_out, ws, s));
 }

@@ -18,7 +18,7 @@ enum : unsigned int {
 //   u32  [d, k]      fp32, as given (CUDA-core paths, row i = U[i, :])
 //   u32t [k, d]      fp32 transpose (CUDA-core reconstruction, coalesced in d)
 //   u32p [d32/2, kp, 2]  fp32, rows of U in pairs, zero past k and d (d32 = d rounded
-//                    up to 32; CUDA-core compress)
+//                    up to 32; CUDA-core compress and projection)
 //   ut16 [n_pad, d]  bf16 U^T, rows >= k zero: B operand of the d -> k contraction
 //   up16 [d, k64]    bf16 U, columns >= k zero: operand of the k -> d expansion
 struct sn_basis {

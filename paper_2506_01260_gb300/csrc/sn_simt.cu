@@ -101,10 +101,10 @@ __device__ __forceinline__ void cp_async_wait_all()
 // has not all of the SMs (a cluster might find no place in it), else the power of two up
 // to 8 with the least (rounds of the grid) x (steps per CTA + 3 for its start + one
 // for each CTA whose partial sums meet), every CTA keeping at least one step.  Among
-// equal costs, the fewest CTAs.  Measured on whole calls, with 1 / 2 / 4 / 8 CTAs (W one
-// step ahead): projection of [2048, 2048] at k = 20 (16 tiles) 74 / 48 / 33 / 37 us, of
-// [2048, 8192] (64 tiles) 92 / 67 / 72 / 90 us; compress of 8192 x 2048 (256 tiles) 31 /
-// 34 / 35 / 43 us.
+// equal costs, the fewest CTAs.  Measured on whole calls, with 1 / 2 / 4 / 8 CTAs:
+// compress of 8192 x 2048 (256 tiles) 31 / 34 / 35 / 43 us; projection at k = 20, when its
+// first pass still loaded W a single step ahead, of [2048, 2048] (16 tiles) 74 / 48 / 33 / 37 us, of
+// [2048, 8192] (64 tiles) 92 / 67 / 72 / 90 us.
 int cluster_split(int64_t tiles, int steps, int sms, int per_sm, cudaStream_t s)
 {
     const int64_t slots = (int64_t)sms * per_sm;
@@ -134,11 +134,10 @@ int cluster_split(int64_t tiles, int steps, int sms, int per_sm, cudaStream_t s)
 // as they lie in shared memory.  At T = 8192, d = 2048, k = 20 (134 and 67 MB read):
 // 42 us with embeddings (3.3 TB/s) and 30 us without, where one output per thread
 // and one pair of shared loads per FMA took 271 and 239 us.  What bounds it is the
-// issue rate of the 7-8 warps that the registers leave on an SM (0.37 a cycle) and
-// the shared loads: 28 passes per 20 cycles of FMAs, since a pass serves equal
-// addresses only where neighbouring lanes share them.  Tiles of 8 tokens a thread
-// (18 passes) need 255 registers and were slower (48 and 30 us), so were chunks of
-// 16 columns at twice the warps (45 us).
+// latency of the 7 warps that the registers leave on an SM, on shared loads for the
+// most part: 0.36 instructions a cycle and scheduler, the shared-memory pipe 37 and 49% busy,
+// the FMA pipe 30 and 36%.  Tiles of 8 tokens a thread need 255 registers and were
+// slower (48 and 30 us), so were chunks of 16 columns at twice the warps (45 us).
 constexpr int CTM = 4;          // tokens per thread
 constexpr int CTOK = 8 * CTM;   // tokens per CTA
 constexpr int CCH = 32;         // columns of d per chunk
@@ -341,7 +340,8 @@ __global__ void __launch_bounds__(CTHREADS) k_simt_compress(const SimtCompress p
 // packed FMA takes two adjacent columns and an element of L twice.  At T = 8192,
 // d = 2048, k = 20: 28 us without and 45 us with embeddings (one column and 8 tokens a
 // thread: 40 and 72 us); the projection's second pass to [2048, 8192] 28 us (98).  The
-// FMA pipe is half busy; the rest is the stores and, with embeddings, the T_fixed rows.
+// FMA pipe is half busy; the rest is the stores and, with embeddings, the T_fixed rows
+// (whose form spills 40 bytes a thread to stay at two CTAs an SM).
 constexpr int ETILE = 128;      // columns per CTA, rows per step of its eight warps
 constexpr int EROWS = 16;       // rows per warp and step
 constexpr int ETHREADS = 256;
@@ -582,8 +582,8 @@ __global__ void __launch_bounds__(FTHREADS) k_simt_expand_few(const SimtExpand p
 // load for 8 packed FMAs.  [2048, 2048] and [2048, 8192] at k = 20: 18 and 29 us (HBM
 // 2.5 and 10, FMA pipe 2.3 and 9 on all SMs), 20 and 35 with W a single step ahead in
 // registers, and 1297 and 1339 with a thread per column that walked all of d with one
-// load of U per FMA.  The FMA pipe is 42% busy: two warps a scheduler issue 0.4 a
-// cycle.  Three CTAs of four warps on an SM were slower (18 and 33 us).
+// load of U per FMA.  The FMA pipe is 38 and 42% busy: two warps a scheduler issue 0.36
+// and 0.39 a cycle.  Three CTAs of four warps on an SM were slower (18 and 33 us).
 constexpr int PROWS = 8;        // rows of W per group and step
 constexpr int PTHREADS = 256;
 constexpr int PSTEPS = 4;       // steps in the ring
@@ -749,7 +749,8 @@ cudaError_t launch_compress_f32(SimtCompress p, bool gather, int sms, cudaStream
     constexpr size_t smem = stage > red ? stage : red;
     const int64_t tiles = (p.T + CTOK - 1) / CTOK;
     const int steps = ((p.d + CCH - 1) / CCH + G - 1) / G;
-    // registers let two (gather) or three CTAs share an SM
+    // registers let two (gather) or three CTAs share an SM for k = 13 .. 32; three or four
+    // fit at other widths, where the split may come out larger than it need be
     p.split = cluster_split(tiles, steps, sms, gather ? 2 : 3, s);
     const unsigned grid = (unsigned)(tiles * p.split);
     void (*const kernel)(SimtCompress) =

@@ -404,9 +404,6 @@ __device__ __forceinline__ void sts128(uint32_t a, uint4 v)
                  "r"(v.w)
                  : "memory");
 }
-__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
-// Two fp32 values -> packed bf16x2 (round-to-nearest-even), `lo` in the low half.
 // c + (bf16 in the low / high half of w), one fp32 rounding, no unpacking
 __device__ __forceinline__ float add_bf16_lo(uint32_t w, float c)
 {
@@ -425,6 +422,7 @@ __device__ __forceinline__ float add_bf16_hi(uint32_t w, float c)
     return r;
 }
 
+// Two fp32 values -> packed bf16x2 (round-to-nearest-even), `lo` in the low half.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 {
     uint32_t r;
